@@ -312,12 +312,14 @@ int eulbfs_set_whole_step(eulbfs_solver* s, int on);
  * steps (0 disables); replays are used when n is a multiple of it. */
 int eulbfs_use_graphs(eulbfs_solver* s, int steps_per_graph);
 
-/* Work-item shape of the stage kernel: each item is a 31-column strip of a
+/* Work-item shape of the stage kernels: each item is a 31-column strip of a
  * domain and a run of its rows.  `rows` (a multiple of 8 in [8, 1024];
- * 0 = 64) is the target height: a domain of ny rows is cut into
- * round(ny / rows) runs (at least one) of nearly equal height, in whole
- * 8-row chunks.  The persistent CTAs claim items from a counter, tallest
- * first.  Results do not depend on it. */
+ * 0 = 128, the default) is the largest target height: a domain of ny rows is
+ * cut into round(ny / rows) runs (at least one) of nearly equal height, in
+ * whole 8-row chunks, or into shorter ones (down to one row) where the batch
+ * has too few cells to fill the GPU with items of that height.  The
+ * persistent CTAs claim items from a counter, tallest first.  Results do not
+ * depend on it. */
 int eulbfs_set_tile(eulbfs_solver* s, int rows);
 
 /* Diagnostics of a caller-held domain state that allocates no device memory.

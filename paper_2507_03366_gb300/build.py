@@ -1,6 +1,6 @@
 """Build libeulbfs.so (sm_103a) in-tree with nvcc.
 
-The translation units (stage kernel, auxiliary kernels, host API, FMA
+The translation units (stage kernels, auxiliary kernels, host API, FMA
 peaks) compile in parallel; the
 result lands in ``paper_2507_03366_gb300/_build/libeulbfs.so``.  Run as a
 module (``python -m paper_2507_03366_gb300.build``) or call ``build()``.
@@ -18,7 +18,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libeulbfs.so")
-SOURCES = ["stage.cu", "kernels.cu", "api.cu", "peaks.cu"]
+SOURCES = ["stage.cu", "stage_short.cu", "kernels.cu", "api.cu", "peaks.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

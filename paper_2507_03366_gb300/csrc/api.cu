@@ -169,6 +169,7 @@ int eulbfs::set_error(int code, const char* msg) { return fail(code, msg); }
 
 constexpr int kMaxTune = 8;   // autotune candidates kept for eulbfs_autotune_report
 constexpr int kTailLevels = 2;   // halvings of the work list's last wave (launches per stage)
+constexpr int kDefaultRows = 128;   // tallest work item unless eulbfs_set_tile says otherwise
 constexpr int kMaxLaunchSteps = 16;   // time steps in one whole-step launch at most
 
 struct eulbfs_solver {
@@ -183,8 +184,9 @@ struct eulbfs_solver {
     int4* d_items = nullptr;       // work items (domain, strip, segment, 0)
     int items_cap = 0;
     int nitems = 0;
+    bool short_items = false;      // the work list is for the short-item kernel
     bool dirty = true;
-    int seg = 64;                  // segment height of a work item (rows)
+    int seg = kDefaultRows;        // tallest work item (rows)
     int sms = 1;
     int grid = 1;
     int* d_flag = nullptr;
@@ -298,13 +300,16 @@ std::vector<unsigned char> consts_image(const std::vector<Dom>& doms, const std:
 // wrapped on periodic axes: those are the items listed here (CSR).
 void build_deps(const eulbfs_solver* s, const std::vector<int4>& items, std::vector<int>& dep) {
     const int n = (int)items.size();
-    std::vector<std::vector<std::vector<int>>> by(s->doms.size());   // [domain][strip] -> items
+    // each strip's items in row order: [domain][strip] -> (y0, item)
+    std::vector<std::vector<std::vector<std::pair<int, int>>>> by(s->doms.size());
     for (int i = 0; i < n; ++i) {
         const int4& t = items[i];
         auto& v = by[t.x];
         if (v.empty()) v.resize(s->doms[t.x].desc.strips);
-        v[t.y].push_back(i);
+        v[t.y].push_back({t.z, i});
     }
+    for (auto& d : by)
+        for (auto& v : d) std::sort(v.begin(), v.end());
     dep.assign(n + 1, 0);
     std::vector<char> mark;
     for (int i = 0; i < n; ++i) {
@@ -331,15 +336,54 @@ void build_deps(const eulbfs_solver* s, const std::vector<int4>& items, std::vec
         }
         for (int sx = 0; sx < d.strips; ++sx) {
             if (!mark[sx]) continue;
-            for (int j : by[t.x][sx]) {
-                const int4& u = items[j];
-                bool hit = false;
-                for (int k = 0; k < niv; ++k) hit |= u.z < iv[k][1] && iv[k][0] < u.w;
-                if (hit) dep.push_back(j);
+            const auto& v = by[t.x][sx];
+            const size_t first = dep.size();
+            for (int k = 0; k < niv; ++k) {
+                // the last item that starts at or below the interval, and on to its end
+                auto it = std::upper_bound(v.begin(), v.end(), std::make_pair(iv[k][0], n));
+                if (it != v.begin()) --it;
+                for (; it != v.end() && it->first < iv[k][1]; ++it)
+                    if (items[it->second].w > iv[k][0] &&
+                        std::find(dep.begin() + first, dep.end(), it->second) == dep.end())
+                        dep.push_back(it->second);
             }
         }
         dep[i + 1] = (int)dep.size() - (n + 1);
     }
+}
+
+struct ItemPlan {
+    bool short_items;   // items of at most kShortRows rows, run by the short-item kernel
+    int rows;           // target rows of an item
+};
+
+// How the active domains' rows are cut into work items.  A stage cannot end
+// before its tallest item does, and an item of many rows is a long serial
+// sweep, so a batch that does not fill the chip is cut finer (s->seg stays the
+// upper limit).  us per step on one GB300, FP32C unless marked:
+//   - the short-item kernel, up to 3.2 items of kShortRows rows per SM, in
+//     items just short enough to give each SM one: 128^2 121 -> 15, 400x200 193 -> 24, 333x251
+//     131 -> 27, 1024x4 27 -> 14; FP64 256x4 135 -> 60, 128^2 1281 -> 113,
+//     256^2 1326 -> 371 (tiled kernel, 8-row items: 31, 37, 34, 27; FP64 135,
+//     201, 392);
+//   - else the tiled kernel with the tallest items that still make 1.8 waves of
+//     its resident CTAs: 512^2 148 -> 64 (8 rows; short items 76), 768^2 169 ->
+//     106 (16 rows; 24: 106, 32: 119), 1024^2 223 -> 168 (32 rows; 24: 176,
+//     16: 192), 24 droplet domains 362 (64 rows; 48: 375, 96: 425).
+ItemPlan plan_items(const eulbfs_solver* s) {
+    if (const char* e = getenv("EULBFS_PLAN")) return ItemPlan{e[0] == 's' && !s->tile_probe, atoi(e + 1)};
+    long long strip_rows = 0;   // rows of all strips
+    for (const Dom& d : s->doms)
+        if (d.active()) strip_rows += (long long)((d.grid.nx + kStripX - 1) / kStripX) * d.grid.ny;
+    // input tiles, and so the probe of their waits, are the tiled kernel's
+    if (!s->tile_probe && strip_rows * 10 <= 32 * s->sms * kShortRows) {
+        const long long rows = (strip_rows + s->sms - 1) / s->sms;
+        return ItemPlan{true, (int)std::min<long long>(kShortRows, std::max(1LL, rows))};
+    }
+    const long long resident = (long long)stage_blocks_per_sm(s->precision) * s->sms;
+    const long long rows = strip_rows * 10 / (18 * resident);
+    const int chunks = (int)std::min<long long>(s->seg / kChunk, std::max(1LL, (rows + kChunk / 2) / kChunk));
+    return ItemPlan{false, chunks * kChunk};
 }
 
 int rebuild(eulbfs_solver* s) {
@@ -371,20 +415,24 @@ int rebuild(eulbfs_solver* s) {
         s->consts_cap = std::max(img.size(), 2 * s->consts_cap);
         CK(cudaMalloc(&s->d_consts, s->consts_cap), "constants array");
     }
-    // work items: each domain's kChunk-row chunks split into round(ny / seg)
-    // runs of nearly equal length; the list runs the tallest items first, so
-    // that the persistent CTAs, which claim items in list order, end on the
-    // shortest
+    const ItemPlan plan = plan_items(s);
+    s->short_items = plan.short_items;
+    // work items: each domain's rows (in whole kChunk-row chunks for the tiled
+    // kernel) split into runs of nearly equal length; the list runs the
+    // tallest items first, so that the persistent CTAs, which claim items in
+    // list order, end on the shortest
     std::vector<int4> items;
     for (int k = 0; k < nd; ++k) {
         Dom& d = s->doms[k];
-        const int chunks = (d.grid.ny + kChunk - 1) / kChunk, per = std::max(1, s->seg / kChunk);
+        const int unit = plan.short_items ? 1 : kChunk;
+        const int chunks = (d.grid.ny + unit - 1) / unit, per = std::max(1, plan.rows / unit);
         d.desc.strips = (d.grid.nx + kStripX - 1) / kStripX;
-        d.desc.segs = std::min(chunks, std::max(1, (chunks + per / 2) / per));
+        d.desc.segs = plan.short_items ? (chunks + per - 1) / per
+                                       : std::min(chunks, std::max(1, (chunks + per / 2) / per));
         if (!d.active()) continue;
         for (int sy = 0; sy < d.desc.segs; ++sy) {
-            const int y0 = (int)((long long)sy * chunks / d.desc.segs) * kChunk;
-            const int y1 = std::min(d.grid.ny, (int)((long long)(sy + 1) * chunks / d.desc.segs) * kChunk);
+            const int y0 = (int)((long long)sy * chunks / d.desc.segs) * unit;
+            const int y1 = std::min(d.grid.ny, (int)((long long)(sy + 1) * chunks / d.desc.segs) * unit);
             for (int sx = 0; sx < d.desc.strips; ++sx) items.push_back(make_int4(k, sx, y0, y1));
         }
     }
@@ -400,7 +448,7 @@ int rebuild(eulbfs_solver* s) {
     bool linked = false;
     for (const int2& l : s->links)
         linked |= l.x < nd && l.y < nd && s->doms[l.x].active() && s->doms[l.y].active();
-    const int tail_levels = s->whole_step && !linked ? 0 : kTailLevels;
+    const int tail_levels = plan.short_items || (s->whole_step && !linked) ? 0 : kTailLevels;
     const int resident = stage_blocks_per_sm(s->precision) * s->sms;
     for (int level = 0; level < tail_levels && (long long)items.size() > 2LL * resident; ++level) {
         std::vector<int4> tail;
@@ -464,11 +512,16 @@ int rebuild(eulbfs_solver* s) {
     }
     // the host vectors die here: make the copies complete before returning
     CK(cudaStreamSynchronize(s->stream), "rebuild sync");
-    const int per_sm = stage_blocks_per_sm(s->precision);
+    const int per_sm = plan.short_items ? short_blocks_per_sm(s->precision) : stage_blocks_per_sm(s->precision);
     s->grid = std::max(1, std::min(s->nitems, per_sm * s->sms));
     drop_graph(s);
     s->dirty = false;
     return EULBFS_OK;
+}
+
+cudaError_t launch_items(const eulbfs_solver* s, const StageLaunch& a) {
+    return s->short_items ? launch_short(s->precision, a, s->grid, s->stream)
+                          : launch_stage(s->precision, a, s->grid, s->stream);
 }
 
 // k time steps on the solver's stream: whole-step launches of up to
@@ -497,7 +550,7 @@ int launch_steps_direct(eulbfs_solver* s, long long k) {
         if (s->fused) {
             a.stages = 3 * steps;
             nvtxRangePushA("eulbfs steps");
-            const cudaError_t e = launch_stage(s->precision, a, s->grid, s->stream);
+            const cudaError_t e = launch_items(s, a);
             nvtxRangePop();
             if (e != cudaSuccess) return cuda_fail(e, "stage kernel launch");
             ++s->launches;
@@ -506,7 +559,7 @@ int launch_steps_direct(eulbfs_solver* s, long long k) {
             for (int st = 0; st < 3; ++st) {
                 a.stage = st;
                 nvtxRangePushA(kStageRange[st]);
-                cudaError_t e = launch_stage(s->precision, a, s->grid, s->stream);
+                cudaError_t e = launch_items(s, a);
                 ++s->launches;
                 // split domains: the stage's output halos from the neighbouring slabs
                 if (e == cudaSuccess && s->nlinks) {
@@ -763,7 +816,7 @@ int eulbfs_domain_progress(const eulbfs_solver* s, int slot, long long* done, lo
 
 int eulbfs_set_tile(eulbfs_solver* s, int rows) {
     if (!s) return fail(EULBFS_EINVAL, "null solver");
-    if (rows == 0) rows = 64;
+    if (rows == 0) rows = kDefaultRows;
     if (rows < kChunk || rows > 1024 || rows % kChunk) return fail(EULBFS_EINVAL, "segment height must be a multiple of 8 in [8, 1024]");
     if (rows != s->seg) {
         s->seg = rows;
@@ -842,7 +895,7 @@ int eulbfs_set_tile_wait_probe(eulbfs_solver* s, int on) {
     if (!s || on < 0 || on > 2) return fail(EULBFS_EINVAL, "null solver or on not 0, 1 or 2");
     s->tile_probe = on == 1 ? 16u : 0u;
     s->dep_probe = on == 2 ? 1 : 0;
-    drop_graph(s);
+    s->dirty = true;   // tiles are only waited on by the tiled kernel: the plan follows the probe
     return EULBFS_OK;
 }
 

@@ -159,6 +159,10 @@ __host__ __device__ inline void fill_consts(const DomainDesc& d, Consts<R>& K) {
 constexpr int kStripX = 31;   // 31 cells -> 32 x-faces per row: one per lane
 constexpr int kChunk = 8;
 constexpr int kStageThreads = 32 * kChunk;
+// The kernel for short work items (stage_short.cu): at most kShortRows rows,
+// which with their halo fit the 16-row ring at once.
+constexpr int kShortRows = 8;
+constexpr int kShortThreads = 512;
 
 // The stage kernel's input tiles: kChunk rows x kTileX columns x all state
 // planes of one buffer, copied into shared memory by a TMA tensor copy.  The
@@ -192,6 +196,9 @@ cudaError_t launch_stage(int precision, const StageLaunch& a, int grid, cudaStre
 // Resident CTAs per SM of the stage kernel (for sizing the persistent grid).
 int stage_blocks_per_sm(int precision);
 size_t stage_smem_bytes(int precision);
+// The same for work items of at most kShortRows rows (any row boundaries).
+cudaError_t launch_short(int precision, const StageLaunch& a, int grid, cudaStream_t s);
+int short_blocks_per_sm(int precision);
 
 // Initial state from primitive fields (device double arrays); *bad is set
 // to 1 if any input value is NaN or Inf.

@@ -42,7 +42,8 @@ class Outcome:
 
     @property
     def latency_s(self) -> float:
-        return self.finished_s - self.arrival_s
+        # a closed loop (realtime=False) may admit a case before its nominal arrival
+        return self.finished_s - min(self.arrival_s, self.admitted_s)
 
 
 @dataclass
