@@ -360,30 +360,34 @@ struct ItemPlan {
 // How the active domains' rows are cut into work items.  A stage cannot end
 // before its tallest item does, and an item of many rows is a long serial
 // sweep, so a batch that does not fill the chip is cut finer (s->seg stays the
-// upper limit).  us per step on one GB300, FP32C unless marked:
-//   - the short-item kernel, up to 3.2 items of kShortRows rows per SM, in
-//     items just short enough to give each SM one: 128^2 121 -> 15, 400x200 193 -> 24, 333x251
-//     131 -> 27, 1024x4 27 -> 14; FP64 256x4 135 -> 60, 128^2 1281 -> 113,
-//     256^2 1326 -> 371 (tiled kernel, 8-row items: 31, 37, 34, 27; FP64 135,
-//     201, 392);
-//   - else the tiled kernel with the tallest items that still make 1.8 waves of
-//     its resident CTAs: 512^2 148 -> 64 (8 rows; short items 76), 768^2 169 ->
-//     106 (16 rows; 24: 106, 32: 119), 1024^2 223 -> 168 (32 rows; 24: 176,
-//     16: 192), 24 droplet domains 362 (64 rows; 48: 375, 96: 425).
+// upper limit).  us per step on one GB300, FP32C unless marked; 64: the height
+// that every batch once had:
+//   - the short-item kernel, up to 4.1 items of kShortRows rows per SM (FP64:
+//     2.6), in items just short enough to give each SM one: 128^2 121 (64) ->
+//     14, 400x200 193 -> 24, 333x251 131 -> 24, 1024x4 27 -> 13; FP64 256x4
+//     135 -> 59, 128^2 1281 -> 110, 256^2 1326 -> 348 (the tiled kernel in
+//     8-row items: 31, 37, 34, 26; FP64 135, 201, 391).  At the limit the two
+//     meet: 384^2 41 (tiled 45), 448^2 54 (53); FP64 256^2 348 (391), 320^2 534
+//     (499).  The FP64 pipe makes a ninth face row per sub-core dearer than
+//     another item: 7 rows at most, 348 (8 rows: 366);
+//   - else the tiled kernel with the tallest items that still make 2.6 waves of
+//     its resident CTAs, up to kDefaultRows: 512^2 148 (64) -> 64 (8 rows), 640^2
+//     165 -> 80 (16), 768^2 171 -> 106 (16), 1024^2 223 -> 176 (24; 32: 168,
+//     16: 192), 16 droplet domains 265 -> 260 (40), 64 domains 941 -> 914 (128;
+//     160: 927).
 ItemPlan plan_items(const eulbfs_solver* s) {
-    if (const char* e = getenv("EULBFS_PLAN")) return ItemPlan{e[0] == 's' && !s->tile_probe, atoi(e + 1)};
+    const bool fp64 = s->precision == EULBFS_FP64;
     long long strip_rows = 0;   // rows of all strips
     for (const Dom& d : s->doms)
         if (d.active()) strip_rows += (long long)((d.grid.nx + kStripX - 1) / kStripX) * d.grid.ny;
     // input tiles, and so the probe of their waits, are the tiled kernel's
-    if (!s->tile_probe && strip_rows * 10 <= 32 * s->sms * kShortRows) {
+    if (!s->tile_probe && strip_rows * 10 <= (fp64 ? 26LL : 41LL) * s->sms * kShortRows) {
         const long long rows = (strip_rows + s->sms - 1) / s->sms;
-        return ItemPlan{true, (int)std::min<long long>(kShortRows, std::max(1LL, rows))};
+        return ItemPlan{true, (int)std::min<long long>(fp64 ? kShortRows - 1 : kShortRows, std::max(1LL, rows))};
     }
-    const long long resident = (long long)stage_blocks_per_sm(s->precision) * s->sms;
-    const long long rows = strip_rows * 10 / (18 * resident);
-    const int chunks = (int)std::min<long long>(s->seg / kChunk, std::max(1LL, (rows + kChunk / 2) / kChunk));
-    return ItemPlan{false, chunks * kChunk};
+    const long long wave = (long long)stage_blocks_per_sm(s->precision) * s->sms * kChunk;
+    const long long chunks = (strip_rows * 10 + 26 * wave - 1) / (26 * wave);
+    return ItemPlan{false, (int)std::min<long long>(s->seg / kChunk, std::max(1LL, chunks)) * kChunk};
 }
 
 int rebuild(eulbfs_solver* s) {

@@ -176,7 +176,8 @@ __device__ __forceinline__ void muc_rows(Core<R>& S, int x0, int r0, int nrows) 
     const P2<R>* C = &S.P.rc[0][0];
     // a slab's halo rows take mu_c in place, except the outermost (never read)
     const int rlo = K.hlo ? 1 - K.hlo : 0, rhi = K.hhi ? K.ny + K.hhi - 1 : K.ny;
-    if (x0 >= kHalo - 1 && x0 + NC - (kHalo - 1) <= K.nx && r0 >= rlo && r0 + nrows <= rhi) {
+    if ((K.per_x || (x0 >= kHalo - 1 && x0 + NC - (kHalo - 1) <= K.nx)) &&
+        (K.per_y || (r0 >= rlo && r0 + nrows <= rhi))) {
         // no wall ghost among these cells: the Laplacian in place
         for (int idx = threadIdx.x; idx < total; idx += NTH) {
             const int rr = idx / NC, cc = 1 + idx - rr * NC;

@@ -13,8 +13,9 @@
 //   - 16 warps instead of 8, so that every face of an item of up to 7 rows
 //     (h x-face rows and h + 1 y-face rows, one per warp) is computed at the
 //     same time instead of x-faces, then y-faces;
-//   - the wait for the neighbouring items of the previous stage polls without
-//     sleeping, and the CTA's next item is claimed while the current one runs.
+//   - the last warp claims the CTA's next item and looks up its neighbours
+//     while the current item's faces run; each warp of the cell update
+//     releases its own rows; the wait for the neighbours polls without sleeping.
 #include <mutex>
 
 #include "stage_device.cuh"
@@ -25,6 +26,7 @@ namespace {
 
 constexpr int NTS = kShortThreads;   // 16 warps
 constexpr int NWS = NTS / 32;
+constexpr int kShortDeps = 64;       // neighbours kept in shared memory (9 one-row items of 3 or 4 strips fit)
 
 template <class R>
 struct ShortSmem : Core<R> {
@@ -32,10 +34,64 @@ struct ShortSmem : Core<R> {
     R wn[Prec<R>::NP][kShortRows][32];
     R ws[Prec<R>::NP][kShortRows][32];
     R frac[kShortRows][32];
-    int cur_domain;
-    int next;      // the CTA's next position in the launch's item sequence
-    int ready;     // the current item's inputs are done
+    // the CTA's next work item, put here by the control warp while the
+    // current one runs: its place in the launch, and what it waits for
+    int4 item;
+    int pos;                  // position in the launch's item sequence (>= its length: no more)
+    int stage, index;         // stage of the launch, index in the work list
+    int ndeps, dep0;          // neighbours, and their offset in dep_idx
+    int dep[kShortDeps];      // the first kShortDeps of them
+    int ready;                // the current item's inputs are done
 };
+
+// An item's done flag counts up to kDone: its updating warps add to it one by
+// one, each after its own stores.
+constexpr int kDone = kShortRows;
+
+// Put item number g of the launch into S (one whole warp).
+template <class R>
+__device__ __forceinline__ void look_up(ShortSmem<R>& S, const StageLaunch& a, int g, int lane) {
+    if (g < a.nitems * a.stages) {
+        const int2 si = stage_item(a, g);
+        const int4 item = a.items[si.y];
+        int d0 = 0, n = 0;
+        if (a.stages > 1 && si.x > 0) {   // one-stage launches are ordered by the kernel boundary
+            d0 = a.dep_off[si.y];
+            n = a.dep_off[si.y + 1] - d0;
+            for (int j = lane; j < min(n, kShortDeps); j += 32) S.dep[j] = a.dep_idx[d0 + j];
+        }
+        if (lane == 0) {
+            S.item = item;
+            S.stage = si.x;
+            S.index = si.y;
+            S.ndeps = n;
+            S.dep0 = d0;
+        }
+    }
+    if (lane == 0) S.pos = g;
+}
+
+// Wait until every item that the current one reads has finished the previous
+// stage (one warp; lanes take one neighbour each).  A bounded wait, as
+// deps_ready of stage_device.cuh, but it polls without sleeping: the next
+// stage starts when the slowest neighbour's flag is seen.
+template <class R>
+__device__ __forceinline__ bool wait_deps(const ShortSmem<R>& S, const StageLaunch& a, int st, int n, int lane) {
+    const int* done = a.done + (size_t)(st - 1) * a.nitems;
+    bool ok = true;
+    for (int j = lane; j < n; j += 32) {
+        const int* f = done + (j < kShortDeps ? S.dep[j] : a.dep_idx[S.dep0 + j]);
+        if (ld_acquire(f) >= kDone) continue;
+        const long long t0 = clock64();
+        while (ld_acquire(f) < kDone)
+            if (clock64() - t0 > (1LL << 31)) { ok = false; break; }
+    }
+    return __all_sync(0xffffffffu, ok);
+}
+
+__device__ __forceinline__ void add_release(int* p, int v) {
+    asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 
 __device__ __forceinline__ void put_cell(float (*p)[kShortRows][32], int r, int l, const SV<float>& w) {
     p[0][r][l] = w.Hh; p[1][r][l] = w.Hl; p[2][r][l] = w.p; p[3][r][l] = w.mx; p[4][r][l] = w.my;
@@ -61,36 +117,32 @@ struct SharedCell {
     __device__ __forceinline__ SV<R> ws() const { return get_cell(S.ws, row, lane); }
 };
 
-// Cell idx of the item's rows with halo: load its raw state.
+// Load and derive cell (gx, gy) into ring column cc; a halo cell outside the
+// domain is mapped through the boundary rules (as load_rows).
 template <class R>
-struct HaloCell {
-    int gx, gy, sx, sy, kx, ky, sdx, sdy;
-};
-
-template <class R>
-__device__ __forceinline__ SV<R> fetch_cell(const Consts<R>& K, const R* in, int gx, int gy, HaloCell<R>& h) {
-    h.gx = gx;
-    h.gy = gy;
-    map_axis(gx, K.nx, K.per_x, XLO, h.sx, h.kx, h.sdx);
-    map_row(K, gy, h.sy, h.ky, h.sdy);
-    return load_state(in, K.plane, (long long)h.sy * K.nx + h.sx + K.off);
-}
-
-template <class R>
-__device__ __forceinline__ void derive_cell(ShortSmem<R>& S, const R* in, const HaloCell<R>& h, const SV<R>& w,
-                                            int cc) {
+__device__ __forceinline__ SV<R> ring_cell(ShortSmem<R>& S, const R* in, int gx, int gy, int cc, bool inside) {
     const Consts<R>& K = S.K;
+    int sx = gx, sy = gy, kx = 0, ky = 0, sdx = XLO, sdy = YLO;
+    if (!inside) {
+        map_axis(gx, K.nx, K.per_x, XLO, sx, kx, sdx);
+        map_row(K, gy, sy, ky, sdy);
+    }
+    const SV<R> w = load_state(in, K.plane, (long long)sy * K.nx + sx + K.off);
     Prim<R> q = derive(K, w);
-    // x sides first, then y (corners), as load_rows
-    if (h.kx) apply_ghost(K, h.sdx, h.kx, true, wall_wetting(K, in, h.sdx, h.sy), q);
-    if (h.ky) apply_ghost(K, h.sdy, h.ky, false, wall_wetting(K, in, h.sdy, h.gx), q);
-    store_prim(S, slot(h.gy), cc, q);
+    if (!inside) {
+        // x sides first, then y (corners)
+        if (kx) apply_ghost(K, sdx, kx, true, wall_wetting(K, in, sdx, sy), q);
+        if (ky) apply_ghost(K, sdy, ky, false, wall_wetting(K, in, sdy, gx), q);
+    }
+    store_prim(S, slot(gy), cc, q);
+    return w;
 }
 
 // One work item: rows [y0, y1) (at most kShortRows) of the strip at x0.
+// `claim`: the control warp's claimed next position, looked up in here.
 template <class R, bool AXI, bool GEN>
 __device__ __forceinline__ void short_item(ShortSmem<R>& S, const StageLaunch& a, const int stage, int x0, int y0,
-                                           int y1) {
+                                           int y1, int claim) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const Consts<R>& K = S.K;
     const R* in = reinterpret_cast<const R*>(K.st[stage]);
@@ -107,14 +159,13 @@ __device__ __forceinline__ void short_item(ShortSmem<R>& S, const StageLaunch& a
         if (stage != 0) wn = load_state(reinterpret_cast<const R*>(K.st[0]), K.plane, c);
     }
     // ... and the rows with their halo
+    const bool inside = x0 >= kHalo && x0 + kStripX + kHalo <= K.nx && y0 - kHalo >= -K.hlo && y1 + kHalo <= K.ny + K.hhi;
     const int total = (rows + 2 * kHalo) * RW;
     for (int idx = tid; idx < total; idx += NTS) {
         const int rr = idx / RW, cc = idx - rr * RW;
-        HaloCell<R> h;
-        const SV<R> w = fetch_cell(K, in, x0 + cc - kHalo, y0 + rr - kHalo, h);
+        const SV<R> w = ring_cell(S, in, x0 + cc - kHalo, y0 + rr - kHalo, cc, inside);
         const int ir = rr - kHalo, ic = cc - kHalo;
         if (ir >= 0 && ir < rows && ic >= 0 && ic < kStripX) put_cell(S.ws, ir, ic, w);
-        derive_cell(S, in, h, w, cc);
     }
     if (upd) {
         S.frac[ur][ul] = fr;
@@ -125,6 +176,7 @@ __device__ __forceinline__ void short_item(ShortSmem<R>& S, const StageLaunch& a
     __syncthreads();
     muc_rows<R, AXI, NTS>(S, x0, y0 - 2, rows + 4);
     __syncthreads();
+    if (warp == NWS - 1) look_up(S, a, __shfl_sync(0xffffffffu, claim, 0), lane);
     // face rows: x-faces of every row, then the y-faces below and above every row
 #pragma unroll 1
     for (int t = warp; t < 2 * rows + 1; t += NWS) {
@@ -158,51 +210,53 @@ __global__ void __launch_bounds__(NTS, sizeof(R) == 4 ? 2 : 1) short_kernel(Stag
     const int tid = threadIdx.x;
     const Consts<R>* consts = static_cast<const Consts<R>*>(a.consts);
     int* const counter = a.work + (a.stages == 1 ? a.stage : 0);
-    if (tid == 0) {
-        S.cur_domain = -1;
-        S.next = atomicAdd(counter, 1);
-    }
-    __syncthreads();
+    const int lane = tid & 31, warp = tid >> 5;
     // items are claimed in order, one ahead, as in stage.cu: every item waits
     // only for items claimed before it
-    while (S.next < a.nitems * a.stages) {
-        const int2 si = stage_item(a, S.next);
-        const int4 item = a.items[si.y];
-        const bool other = item.x != S.cur_domain;
-        __syncthreads();                 // every thread has read S.next and S.cur_domain
-        int claimed = 0;
-        if (tid == 0) claimed = atomicAdd(counter, 1);
-        if (other) {
-            const unsigned* src = reinterpret_cast<const unsigned*>(consts + item.x);
+    if (warp == NWS - 1) {
+        int g = 0;
+        if (lane == 0) g = atomicAdd(counter, 1);
+        look_up(S, a, __shfl_sync(0xffffffffu, g, 0), lane);
+    }
+    __syncthreads();
+    int domain = -1;
+    // From here to the barrier below, warps may still be in the previous
+    // item's cell update: only S.ready is written.  The look-up of the item
+    // after this one comes behind two more barriers.
+    while (S.pos < a.nitems * a.stages) {
+        const int4 item = S.item;
+        const int st = S.stage, index = S.index;
+        if (item.x != domain) {
+            if (domain >= 0) __syncthreads();   // the previous item is done with S.K
+            domain = item.x;
+            const unsigned* src = reinterpret_cast<const unsigned*>(consts + domain);
             unsigned* dst = reinterpret_cast<unsigned*>(&S.K);
             for (int k = tid; k < (int)(sizeof(Consts<R>) / 4); k += NTS) dst[k] = src[k];
-            if (tid == 0) S.cur_domain = item.x;
         }
-        if (a.stages > 1 && si.x > 0 && tid < 32) {
-            const bool ready = deps_ready(a, si.x, si.y, tid, true, 0);
-            if (tid == 0) S.ready = ready;
-        } else if (tid == 0) {
-            S.ready = 1;
+        if (warp == 0) {
+            const bool ready = S.ndeps == 0 || wait_deps(S, a, st, S.ndeps, lane);
+            if (lane == 0) S.ready = ready;
         }
-        __syncthreads();                 // S.K, S.ready
+        __syncthreads();                 // S.K, S.ready; the previous item is done with shared memory
         if (!S.ready) {                  // a bounded wait gave up: report it and stop
             if (tid == 0) atomicOr(a.flag, 2);
             return;
         }
+        int claim = 0;
+        if (tid == NTS - 32) claim = atomicAdd(counter, 1);
         const int x0 = item.y * kStripX;
-        const int stage = si.x % 3;
+        const int stage = st % 3;
         if (S.K.gen) {
-            if (S.K.axi) short_item<R, true, true>(S, a, stage, x0, item.z, item.w);
-            else short_item<R, false, true>(S, a, stage, x0, item.z, item.w);
+            if (S.K.axi) short_item<R, true, true>(S, a, stage, x0, item.z, item.w, claim);
+            else short_item<R, false, true>(S, a, stage, x0, item.z, item.w, claim);
         } else {
-            if (S.K.axi) short_item<R, true, false>(S, a, stage, x0, item.z, item.w);
-            else short_item<R, false, false>(S, a, stage, x0, item.z, item.w);
+            if (S.K.axi) short_item<R, true, false>(S, a, stage, x0, item.z, item.w, claim);
+            else short_item<R, false, false>(S, a, stage, x0, item.z, item.w, claim);
         }
-        if (tid == 0) S.next = claimed;
-        __syncthreads();                 // every thread's stores of this item; S.next
-        if (a.stages > 1 && tid == 0 && !a.dep_probe) {
-            __threadfence();
-            atomicExch(a.done + (size_t)si.x * a.nitems + si.y, 1);
+        const int rows = item.w - item.z;
+        if (a.stages > 1 && warp < rows && !a.dep_probe) {
+            __syncwarp();                // every lane's stores of this row
+            if (lane == 0) add_release(a.done + (size_t)st * a.nitems + index, warp == 0 ? kDone + 1 - rows : 1);
         }
     }
 }
