@@ -70,7 +70,9 @@ struct Consts {
     //    printed {cp_s, 0, cp_g, cp_l - cp_g};
     //  - face {Q, C_ref / 6, 6 / C_ref, tau_g - 1/2}; cell {kv, g_x, g_y, 1 / dt}
     //    and {2 beta, kappa, dt, dt_f}
-    Q4<R> mcp, mrho, mlam, mmu, enth, enthc, facec, cellc, cellc2;
+    //  - faces with dt_s = 0.5: {3 Q, 3 Q / 4, C_ref / 6, 6 / C_ref}
+    Q4<R> mcp, mrho, mlam, mmu, enth, enthc, facec, cellc, cellc2, facek;
+    alignas(2 * sizeof(R)) R facet[2];   // (1 - t, t / 6) of t = tau_g - 1/2
     // H_l = C_p^liq hl[0] + hl[1]: R1 {T_l, L}, as printed {0, cp_l T_l + L}
     alignas(2 * sizeof(R)) R hl[2];
     R printed;                 // 1 with Eq. 5-7 as printed, 0 with reading R1
@@ -126,6 +128,9 @@ __host__ __device__ inline void fill_consts(const DomainDesc& d, Consts<R>& K) {
     K.facec = make_q4<R>(d.Qg, d.Cref / 6.0, 6.0 / d.Cref, d.tau_g - 0.5);
     K.cellc = make_q4<R>(d.kv, d.gx, d.gy, 1.0 / d.dt);
     K.cellc2 = make_q4<R>(2.0 * d.beta, d.kappa, d.dt, d.dts[1]);
+    K.facek = make_q4<R>(3.0 * d.Qg, 0.75 * d.Qg, d.Cref / 6.0, 6.0 / d.Cref);
+    K.facet[0] = (R)(1.5 - d.tau_g);
+    K.facet[1] = (R)((d.tau_g - 0.5) / 6.0);
     for (int k = 0; k < 3; ++k) K.cp[k] = (R)d.cp[k];
     K.L = (R)d.L; K.Ts = (R)d.Ts; K.Tl = (R)d.Tl;
     K.four_over_xi = (R)d.four_over_xi;

@@ -220,12 +220,18 @@ struct FaceIdx { int L, R, LL, RR, Lp, Lm, Rp, Rm; };
 template <class R>
 struct FaceFlux { R Fh, Fp, Fmn, Fmt, Fc, un; };
 
-// Reconstruction pieces of one field: the cell values l, r, the face value
-// o0 (mean of the two one-sided reconstructions l + (r - ll)/4 and
-// r - (rr - l)/4, i.e. 5/8 (l + r) - 1/8 (ll + rr)) and the central
-// t-differences dtl, dtr of the two cells (half-cell t-step = dt / 4).
+// Reconstruction pieces of one field: the cell values l, r, eight times the
+// face value f8 (the face value is the mean of the two one-sided
+// reconstructions l + (r - ll)/4 and r - (rr - l)/4, i.e. 5/8 (l + r) -
+// 1/8 (ll + rr); powers of two are left to the constants it meets) and the
+// central t-differences dtl, dtr of the two cells (half-cell t-step = dt / 4).
 template <class R>
-struct Rec { R l, r, o0, dtl, dtr; };
+struct Rec { R l, r, f8, dtl, dtr; };
+
+template <class R>
+__device__ __forceinline__ R face_value8(R l, R r, R ll, R rr) {
+    return fma(R(5), l + r, -(ll + rr));
+}
 
 template <class R>
 __device__ __forceinline__ R face_value(R l, R r, R ll, R rr) {
@@ -237,7 +243,7 @@ __device__ __forceinline__ Rec<R> rec_of(R l, R r, R ll, R rr, R lp, R lm, R rp,
     Rec<R> z;
     z.l = l;
     z.r = r;
-    z.o0 = face_value(l, r, ll, rr);
+    z.f8 = face_value8(l, r, ll, rr);
     z.dtl = lp - lm;
     z.dtr = rp - rm;
     return z;
@@ -260,47 +266,59 @@ __device__ __forceinline__ void face_value2(const P2<R>* f, const FaceIdx& x, R&
     b = face_value(l.y, r.y, ll.y, rr.y);
 }
 
-// The nonlinear parts of the equilibrium moments over the surrounding points
-// of one side column of a face: the points x_f - e_a dt_s with e_n = sn
-// (+1: the L cell, points 1, 5, 8; -1: the R cell, points 3, 6, 7).  The
-// column's centre point (e_t = 0) takes the cell values; its t-points
-// (e_t = +1 / -1) the cell value minus / plus a quarter of the central
-// t-difference.  With q = e.u + 3/2 (e.u)^2 - 1/2 u^2 (cs^2 = 1/3):
-//   centre:   q = sn u_n + u_n^2 - u_t^2 / 2
-//   t-points: q = e.u (1 + e.u) + e_n e_t u_n u_t
-// Returned: at the centre rho q, C u_n, q, C_p T q; over the t-points the sum
-// (e_t = +1 plus e_t = -1) of rho q, C e.u, q and C_p T q, and the difference
-// (+1 minus -1) of rho q and q.
+// The same times eight.
 template <class R>
-struct SideSums { R f0, c0, q0, h0, fs, fd, cs, qs, qd, hs; };
+__device__ __forceinline__ void face_value8_2(const P2<R>* f, const FaceIdx& x, R& a, R& b) {
+    const P2<R> l = f[x.L], r = f[x.R], ll = f[x.LL], rr = f[x.RR];
+    a = face_value8(l.x, r.x, ll.x, rr.x);
+    b = face_value8(l.y, r.y, ll.y, rr.y);
+}
+
+// What one side column of a face adds to its moments: the points
+// x_f - e_a dt_s with e_n = SN (+1: the L cell, points 1, 5, 8; -1: the R cell,
+// points 3, 6, 7).  The column's centre point (e_t = 0) takes the cell values;
+// its t-points (e_t = +1 / -1) the cell value minus / plus a quarter d of the
+// central t-difference.  With q = e.u + 3/2 (e.u)^2 - 1/2 u^2 (cs^2 = 1/3):
+//   centre:   q0 = SN u_n + u_n^2 - u_t^2 / 2
+//   t-points: q = e.u (1 + e.u) + e_n e_t u_n u_t, where with
+//             A = SN u_n - d u_t, B = u_t - SN d u_n:  e.u = A + B and A - B,
+// so that the two t-points' half sum and half difference of q are
+//   hq = A + A^2 + B^2 - SN (u_n d u_t + d u_n u_t)
+//   hd = B (1 + 2 A) + SN (u_n u_t + d u_n d u_t),
+// and the half sum / difference of (f - / + df) q are f hq - df hd and
+// f hd - df hq.  The weights of the centre (1/9) and the t-points (1/36, in pairs
+// 1/18) then meet as V = 2 q0 + hq = 18 sum w q.  Per side, scaled:
+//   X = rho V - d rho hd         18 x its part of sum f, of +- sum e_n f
+//   F = rho hd - d rho hq        18 x its part of sum e_t f
+//   G = C (2 SN u_n + A) - d C B    6 x its part of sum g, of +- sum e_n g
+//   H = C_p T V + d C_p d T hq - (C_p d T + d C_p T) hd    6 x its part of +- sum e_n h
+// The parts linear in p, mu_c and T stay out of them, so that the flux takes
+// their differences across the face exactly.
+// Folding the weights into V and so into X, G and H takes a face from about 237
+// to 191 FP operations besides its division (against the t-points one by one and
+// each moment from its own sums).  us per step: FP64, bound by its pipe, 16
+// domains 6460 -> 5760, 256^2 348 -> 316; FP32C, bound by issue, 64 domains 1023
+// -> 977, 16 domains 260 -> 251, 512^2 63.6 -> 60.9.  Constants like 1/6 are a
+// biased 3e-8 in FP32: none stands on an undivided advective or conductive flux.
+template <class R>
+struct SideTerms { R X, V, hd, F, G, H; };
 
 template <class R, int SN>
-__device__ __forceinline__ SideSums<R> side_sums(R un, R ut, R rho, R C, R T, R cp, R dun, R dut, R drho, R dC,
-                                                 R dT, R dcp) {
-    SideSums<R> s;
+__device__ __forceinline__ SideTerms<R> side_terms(R un, R ut, R rho, R C, R T, R cp, R dun, R dut, R drho, R dC,
+                                                   R dT, R dcp) {
+    constexpr R sg = SN > 0 ? R(1) : R(-1);
     const R sun = SN > 0 ? un : -un;
-    s.q0 = fma(un, un, fma(R(-0.5) * ut, ut, sun));
-    s.f0 = rho * s.q0;
-    s.c0 = C * un;
-    s.h0 = (cp * T) * s.q0;
-    // e_t = +1: value - d/4; e_t = -1: value + d/4
-    const R unp = fma(R(-0.25), dun, un), unm = fma(R(0.25), dun, un);
-    const R utp = fma(R(-0.25), dut, ut), utm = fma(R(0.25), dut, ut);
-    const R eup = (SN > 0 ? unp : -unp) + utp;
-    const R eum = (SN > 0 ? unm : -unm) - utm;
-    const R qp = fma(SN > 0 ? unp : -unp, utp, fma(eup, eup, eup));      // e_n e_t = sn
-    const R qm = fma(SN > 0 ? -unm : unm, utm, fma(eum, eum, eum));      // e_n e_t = -sn
-    const R rp = fma(R(-0.25), drho, rho), rm = fma(R(0.25), drho, rho);
-    const R am = rm * qm;
-    s.fs = fma(rp, qp, am);
-    s.fd = fma(rp, qp, -am);
-    const R Cp_ = fma(R(-0.25), dC, C), Cm_ = fma(R(0.25), dC, C);
-    s.cs = fma(Cp_, eup, Cm_ * eum);
-    s.qs = qp + qm;
-    s.qd = qp - qm;
-    const R hp = fma(R(-0.25), dcp, cp) * fma(R(-0.25), dT, T);
-    const R hm = fma(R(0.25), dcp, cp) * fma(R(0.25), dT, T);
-    s.hs = fma(hp, qp, hm * qm);
+    const R A = fma(R(-0.25), dut, sun), B = fma(R(-0.25) * sg, dun, ut);
+    const R hq = fma(R(-0.25) * sg, fma(dun, ut, un * dut), fma(B, B, fma(A, A, A)));
+    SideTerms<R> s;
+    s.hd = fma(R(1.0 / 16.0) * sg, dun * dut, fma(sun, ut, fma(R(2), A, R(1)) * B));
+    s.V = fma(R(2), fma(un, un, fma(R(-0.5) * ut, ut, sun)), hq);
+    const R dr = R(0.25) * drho;
+    s.X = fma(rho, s.V, -(dr * s.hd));
+    s.F = fma(rho, s.hd, -(dr * hq));
+    s.G = fma(C, fma(R(2) * sg, un, A), -((R(0.25) * dC) * B));
+    const R c4 = R(0.25) * dcp, t4 = R(0.25) * dT;
+    s.H = fma(-fma(c4, T, cp * t4), s.hd, fma(c4 * t4, hq, (cp * T) * s.V));
     return s;
 }
 
@@ -308,94 +326,80 @@ __device__ __forceinline__ SideSums<R> side_sums(R un, R ut, R rho, R C, R T, R 
 //
 // The face equilibria enter only through their closed moments (C_p T u_n,
 // cs^2 (p + rho u_n^2), cs^2 rho u_n u_t, C u_n; Eq. 11 and the moments of
-// Eq. 29, 42).  The sums over the surrounding points x_f - e_a dt_s are
-// split into their parts linear in one reconstructed field, which have
-// closed forms because the reconstruction is linear (the t-offsets cancel in
-// pairs):
+// Eq. 29, 42).  The sums over the surrounding points x_f - e_a dt_s go by
+// columns of equal e_n: the two side columns (side_terms) and the face column
+// e_n = 0.  The parts linear in one reconstructed field have closed forms,
+// because the reconstruction is linear (the t-offsets cancel in pairs):
 //   sum w p = 2/3 p_0 + (p_L + p_R)/6          sum e_n w p = (p_L - p_R)/6
 //   sum e_t w p = -(dp_L + dp_R)/24             sum e_n e_t w p = (dp_R - dp_L)/72
 //   sum_{e_n != 0} w p = (p_L + p_R)/6
 //   mu_c part of sum g = Q ((mu_L + mu_R)/2 - mu_0), of sum e_n g = Q (mu_L - mu_R)/2
 //   C_ref T part of sum e_n h = C_ref (T_L - T_R)/6
-// (dp = central t-difference), and the nonlinear parts (rho q, C e.u,
-// C_p T q, q), which are summed over the points by columns of equal e_n
-// (side_sums above, and the face column e_n = 0 below) so that each sign
-// pattern of the moments is one sum or difference of column sums.
+// (dp = central t-difference).  Face-column values and t-steps are all carried
+// times eight (f8, and the sum of the two cells' t-differences), so its terms
+// come times 64 and, with rho, 512; the constants below undo that.
 //
 // Axisymmetric domains (reading R24): the face pressure is advanced with the
 // axisymmetric mass source -rho cs^2 u_r / r as well, streamed with weight
 // w_a over dt_s.  Of the fluxes only the normal momentum flux changes, by
 // cs^2 dt_s (-rho_f cs^2 u_r / r) = -rho_f u_r / (18 r) with the face values;
 // inv_r = 1 / r of the face (0 on the axis, where the face area is zero).
-//
-// The arithmetic is written for a value type T (the working precision) and a
-// source Src of the reconstruction pieces (RingFace: one face of the ring).
-template <class T, class R, bool AXI, class Src>
-__device__ __forceinline__ FaceFlux<T> face_math(const Q4<R>& fc, const Src& src, T inv_r) {
-    Rec<T> n, t, rho, C, T_, cp;
+template <class R, bool AXI, class Src>
+__device__ __forceinline__ FaceFlux<R> face_math(const Consts<R>& K, const Src& src, R inv_r) {
+    const Q4<R> fc = ld4(K.facek);   // 3 Q, 3 Q / 4, C_ref / 6, 6 / C_ref
+    Rec<R> n, t, rho, C, T, cp, p, muc;
     src.vel(n, t);               // normal and tangential velocity
     src.rc(rho, C);
-    src.tc(T_, cp);
+    src.tc(T, cp);
+    const SideTerms<R> L = side_terms<R, 1>(n.l, t.l, rho.l, C.l, T.l, cp.l, n.dtl, t.dtl, rho.dtl, C.dtl, T.dtl,
+                                            cp.dtl);
+    const SideTerms<R> S = side_terms<R, -1>(n.r, t.r, rho.r, C.r, T.r, cp.r, n.dtr, t.dtr, rho.dtr, C.dtr, T.dtr,
+                                             cp.dtr);
 
-    // side columns: L (points 1, 5, 8) and R (points 3, 6, 7)
-    const SideSums<T> L = side_sums<T, 1>(n.l, t.l, rho.l, C.l, T_.l, cp.l, n.dtl, t.dtl, rho.dtl, C.dtl, T_.dtl,
-                                          cp.dtl);
-    const SideSums<T> Rs = side_sums<T, -1>(n.r, t.r, rho.r, C.r, T_.r, cp.r, n.dtr, t.dtr, rho.dtr, C.dtr, T_.dtr,
-                                            cp.dtr);
+    // face column (e_n = 0): point 0 at the face value, points 2 (e_t = +1) and
+    // 4 (e_t = -1) shifted by the mean t-step st = (dt_L + dt_R) / 8; there
+    // q = e_t u_t + u_t^2 - u_n^2 / 2 and at point 0 q = -u^2 / 2.  hs, hd: half
+    // sum and half difference of q at 2 and 4, times 64
+    const R sn = n.dtl + n.dtr, st = t.dtl + t.dtr, sr = rho.dtl + rho.dtr, sc = C.dtl + C.dtr;
+    const R a = n.f8 * n.f8, b = t.f8 * t.f8;
+    const R hs = fma(R(-0.5), fma(sn, sn, a), fma(R(-8), st, fma(st, st, b)));
+    const R hd = fma(n.f8, sn, fma(R(-2), st, R(8)) * t.f8);
+    const R G0 = fma(rho.f8, hs - (a + b), -(sr * hd));   // 512 x (half the sum of rho q at 2 and 4, less rho u^2 of point 0)
+    const R Gt = fma(rho.f8, hd, -(sr * hs));             // 512 x half the difference of rho q
+    const R cc = fma(C.f8, st, sc * t.f8);                // -32 x the sum of C e.u at 2 and 4
 
-    // face column (e_n = 0): point 0 at the face value, points 2 (e_t = +1)
-    // and 4 (e_t = -1) shifted by the mean t-step; there
-    // q = e_t u_t + u_t^2 - u_n^2 / 2, and at point 0 q = -u^2 / 2
-    const T stn = T(0.125) * (n.dtl + n.dtr), stt = T(0.125) * (t.dtl + t.dtr);
-    const T str = T(0.125) * (rho.dtl + rho.dtr), stc = T(0.125) * (C.dtl + C.dtr);
-    const T un2 = n.o0 - stn, un4 = n.o0 + stn, ut2 = t.o0 - stt, ut4 = t.o0 + stt;
-    const T q2 = fma(ut2, ut2, fma(T(-0.5) * un2, un2, ut2));
-    const T q4 = fma(ut4, ut4, fma(T(-0.5) * un4, un4, -ut4));
-    const T a4 = (rho.o0 + str) * q4;
-    const T f24s = fma(rho.o0 - str, q2, a4);     // rho q at 2 plus at 4
-    const T f24d = fma(rho.o0 - str, q2, -a4);    // rho q at 2 minus at 4
-    const T c24 = fma(C.o0 - stc, ut2, -((C.o0 + stc) * ut4));   // C e.u at 2 plus at 4
-    const T rho_f = rho.o0;
-    const T ruu0 = rho_f * fma(n.o0, n.o0, t.o0 * t.o0);       // -2 rho q at point 0
-
-    Rec<T> p, muc;
+    // Eq. 56 and the moments of the surrounding equilibria
     src.pm(p, muc);
-    T lamf, muf;
-    src.lm(lamf, muf);
-    const T fQ = T(fc.x), fC = T(fc.y), fI = T(fc.z);   // Q, C_ref / 6, 6 / C_ref; fc.w = tau_g - 1/2
-
-    // Eq. 56 and the moments of the surrounding equilibria; weights 4/9, 1/9
-    // (e_n or e_t zero) and 1/36 (diagonal)
-    const T w1 = T(1.0 / 9.0), w5 = T(1.0 / 36.0);
-    const T pf = T(2.0 / 3.0) * p.o0 + T(1.0 / 6.0) * (p.l + p.r) - T(2.0 / 9.0) * ruu0 +
-                 w1 * ((L.f0 + Rs.f0) + f24s) + w5 * (L.fs + Rs.fs);
-    const T mn = T(1.0 / 6.0) * (p.l - p.r) + w1 * (L.f0 - Rs.f0) + w5 * (L.fs - Rs.fs);
-    const T mt = T(-1.0 / 24.0) * (p.dtl + p.dtr) + w1 * f24d + w5 * (L.fd + Rs.fd);
-    const T Cf = C.o0 + fQ * (T(0.5) * (muc.l + muc.r) - muc.o0) + T(1.0 / 3.0) * ((L.c0 - Rs.c0) + c24) +
-                 T(1.0 / 12.0) * (L.cs + Rs.cs);
-    const T Sg = T(0.5) * fQ * (muc.l - muc.r) + T(1.0 / 3.0) * (L.c0 + Rs.c0) + T(1.0 / 12.0) * (L.cs - Rs.cs);
-    const T Sh = fC * (T_.l - T_.r) + T(1.0 / 3.0) * (L.h0 - Rs.h0) + T(1.0 / 12.0) * (L.hs - Rs.hs);
-    const T Snn_p = T(1.0 / 6.0) * (p.l + p.r);
-    const T Snt_p = T(1.0 / 72.0) * (p.dtr - p.dtl);
-    const T Snn_q = w1 * (L.q0 + Rs.q0) + w5 * (L.qs + Rs.qs);
-    const T Snt_q = w5 * (L.qd - Rs.qd);
+    R lam8, mu8;
+    src.lm(lam8, mu8);
+    const R ps = p.l + p.r;
+    const R mn = fma(R(3), p.l - p.r, L.X - S.X);                                                // 18 sum e_n f
+    const R pf = fma(R(1.5), p.f8, fma(R(3), ps, fma(R(1.0 / 128.0), G0, L.X + S.X)));           // 18 p_f
+    const R mt = fma(R(-0.75), p.dtl + p.dtr, fma(R(1.0 / 128.0), Gt, L.F + S.F));               // 18 sum e_t f
+    const R Cf = fma(R(1.0 / 6.0), fma(R(-1.0 / 16.0), cc, fma(fc.y, fma(R(4), muc.l + muc.r, -muc.f8), L.G + S.G)),
+                     R(0.125) * C.f8);                                                           // C_f
+    const R gn = fma(fc.x, muc.l - muc.r, L.G - S.G);                                            // 6 sum e_n g
     // rho_f cs^2 u_f = sum e f^eq (Eq. 56); tau from the face properties (R9)
-    const T irf = wdiv(T(1), rho_f);
-    const T unf = T(3) * mn * irf, utf = T(3) * mt * irf;
-    const T th = fI * lamf * irf;                // tau_h - 0.5 = lambda / (rho C_ref cs^2 dt_s)
-    const T tf = T(6) * muf * irf;               // tau_f - 0.5 = mu / (rho cs^2 dt_s)
-    const T tg = T(fc.w);
-    const T cs2 = T(1.0 / 3.0);
-    FaceFlux<T> F;
+    const R ir = wdiv(R(1), rho.f8);
+    const R i43 = fma(R(1.0 / 3.0), ir, ir);              // 4/3 ir (a rounded 4/3 would bias every advective flux by 3e-8 in FP32)
+    const R un = mn * i43, ut = mt * i43;
+    const R th = fc.w * (lam8 * ir);                      // tau_h - 0.5 = lambda / (rho C_ref cs^2 dt_s)
+    const R tf = R(6) * (mu8 * ir);                       // tau_f - 0.5 = mu / (rho cs^2 dt_s)
+    const R ru = rho.f8 * un;                             // 8 rho_f u_n
+    FaceFlux<R> F;
     // h* = (1.5 - tau) h^eq(x_f) + (tau - 0.5) h^eq(x_f - e dt_s) (Eq. 13, 16)
-    F.Fh = (T(1) - th) * (cp.o0 * T_.o0) * unf + th * Sh;
-    F.Fp = mn;                                    // sum e_n f^eq(x_f) = rho_f cs^2 u_n,f
+    const R fh = R(1.0 / 64.0) * ((cp.f8 * T.f8) * un);
+    F.Fh = fma(th, fma(fc.z, T.l - T.r, fma(R(1.0 / 6.0), L.H - S.H, -fh)), fh);
+    F.Fp = R(1.0 / 18.0) * mn;                            // sum e_n f^eq(x_f) = rho_f cs^2 u_n,f
     // f* = (1.5 - tau_f) f^eq(x_f) + (tau_f - 0.5) f^eq-m (Eq. 35, 37 with R3)
-    F.Fmn = (T(1) - tf) * cs2 * (pf + rho_f * unf * unf) + tf * (Snn_p + rho_f * Snn_q);
-    F.Fmt = (T(1) - tf) * cs2 * rho_f * unf * utf + tf * (Snt_p + rho_f * Snt_q);
-    F.Fc = (T(1) - tg) * Cf * unf + tg * Sg;     // Eq. 44, 46
-    F.un = unf;
-    if (AXI) F.Fmn += T(-1.0 / 18.0) * rho_f * src.radial(n.o0, t.o0) * inv_r;
+    const R nn = fma(R(2.25), ru * un, pf);               // 54 cs^2 (p_f + rho_f u_n^2)
+    F.Fmn = R(1.0 / 54.0) * fma(tf, fma(R(0.375), rho.f8 * (L.V + S.V), R(9) * ps) - nn, nn);
+    const R nt = ru * ut;                                 // 24 cs^2 rho_f u_n u_t
+    const R ns = fma(R(2), p.dtr - p.dtl, rho.f8 * (L.hd - S.hd));   // 144 x f^eq-m's
+    F.Fmt = R(1.0 / 24.0) * fma(tf, fma(R(1.0 / 6.0), ns, -nt), nt);
+    F.Fc = fma(K.facet[0], Cf * un, K.facet[1] * gn);       // Eq. 44, 46
+    F.un = un;
+    if (AXI) F.Fmn = fma(R(-1.0 / 1152.0) * rho.f8, src.radial(n.f8, t.f8) * inv_r, F.Fmn);
     return F;
 }
 
@@ -414,7 +418,7 @@ struct RingFace {
     __device__ __forceinline__ void rc(Rec<R>& a, Rec<R>& b) const { rec2(&P.rc[0][0], x, a, b); }
     __device__ __forceinline__ void tc(Rec<R>& a, Rec<R>& b) const { rec2(&P.tc[0][0], x, a, b); }
     __device__ __forceinline__ void pm(Rec<R>& a, Rec<R>& b) const { rec2(&P.pm[0][0], x, a, b); }
-    __device__ __forceinline__ void lm(R& a, R& b) const { face_value2(&P.lm[0][0], x, a, b); }
+    __device__ __forceinline__ void lm(R& a, R& b) const { face_value8_2(&P.lm[0][0], x, a, b); }
     __device__ __forceinline__ R radial(R n0, R t0) const { return normal_is_r ? n0 : t0; }
 };
 
@@ -422,7 +426,7 @@ template <class R, bool AXI>
 __device__ __forceinline__ FaceFlux<R> face_flux(const Consts<R>& K, const Ring<R>& P, const FaceIdx& x, bool normal_x,
                                                  bool normal_is_r, R inv_r) {
     const RingFace<R> src{P, x, normal_x, normal_is_r};
-    return face_math<R, R, AXI>(ld4(K.facec), src, inv_r);
+    return face_math<R, AXI>(K, src, inv_r);
 }
 
 
