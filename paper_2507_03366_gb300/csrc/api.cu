@@ -362,29 +362,48 @@ struct ItemPlan {
 // sweep, so a batch that does not fill the chip is cut finer (s->seg stays the
 // upper limit).  us per step on one GB300, FP32C unless marked; 64: the height
 // that every batch once had:
-//   - the short-item kernel, up to 4.1 items of kShortRows rows per SM (FP64:
-//     2.6), in items just short enough to give each SM one: 128^2 121 (64) ->
-//     14, 400x200 193 -> 24, 333x251 131 -> 24, 1024x4 27 -> 13; FP64 256x4
-//     135 -> 59, 128^2 1281 -> 110, 256^2 1326 -> 348 (the tiled kernel in
-//     8-row items: 31, 37, 34, 26; FP64 135, 201, 391).  At the limit the two
-//     meet: 384^2 41 (tiled 45), 448^2 54 (53); FP64 256^2 348 (391), 320^2 534
-//     (499).  The FP64 pipe makes a ninth face row per sub-core dearer than
-//     another item: 7 rows at most, 348 (8 rows: 366);
+//   - the short-item kernel, up to 4.1 items of kShortRows rows per SM: 128^2
+//     121 (64) -> 14.3, 400x200 193 -> 23, 333x251 131 -> 23, 1024x4 27 -> 12.9;
+//     FP64 256x4 135 -> 50, 128^2 1281 -> 115, 256^2 1326 -> 292 (the tiled
+//     kernel in 8-row items: 31, 37, 34, 26; FP64 135, 192, 340).  At the limit
+//     the two meet: 384^2 39 (tiled 43), 448^2 53 (50); FP64 384^2 590 (611);
 //   - else the tiled kernel with the tallest items that still make 2.6 waves of
 //     its resident CTAs, up to kDefaultRows: 512^2 148 (64) -> 64 (8 rows), 640^2
 //     165 -> 80 (16), 768^2 171 -> 106 (16), 1024^2 223 -> 176 (24; 32: 168,
 //     16: 192), 16 droplet domains 265 -> 260 (40), 64 domains 941 -> 914 (128;
 //     160: 927).
+// The height of short items: the one with the least work for the busiest SM.  An
+// item of h rows costs as b + h (a stage of one FP64 item keeps its SM's pipe
+// busy for about 8 + 9 h thousand clocks, whoever shares the SM; fitted for
+// FP32C), so 203 items on 152 SMs take as long as 304; beyond two per SM, items
+// are claimed as SMs get free.  us per step: 200^2 FP64 262 with 7 rows (203
+// items), 194 with 4 (350); FP32C 20.7 with 8 rows (175 items), 17.9 with 5 (280).
+int short_rows(const eulbfs_solver* s, bool fp64) {
+    const int most = fp64 ? kShortRows64 : kShortRows;
+    const double b = fp64 ? 0.9 : 2.8;
+    int best = 1;
+    double least = 0.0;
+    for (int h = 1; h <= most; ++h) {
+        long long n = 0;
+        for (const Dom& d : s->doms)
+            if (d.active()) n += (long long)((d.grid.nx + kStripX - 1) / kStripX) * ((d.grid.ny + h - 1) / h);
+        const double per_sm = n <= 2LL * s->sms ? (double)((n + s->sms - 1) / s->sms) : (double)n / s->sms;
+        const double work = per_sm * (b + h);
+        if (h == 1 || work < least) {
+            best = h;
+            least = work;
+        }
+    }
+    return best;
+}
+
 ItemPlan plan_items(const eulbfs_solver* s) {
     const bool fp64 = s->precision == EULBFS_FP64;
     long long strip_rows = 0;   // rows of all strips
     for (const Dom& d : s->doms)
         if (d.active()) strip_rows += (long long)((d.grid.nx + kStripX - 1) / kStripX) * d.grid.ny;
     // input tiles, and so the probe of their waits, are the tiled kernel's
-    if (!s->tile_probe && strip_rows * 10 <= (fp64 ? 26LL : 41LL) * s->sms * kShortRows) {
-        const long long rows = (strip_rows + s->sms - 1) / s->sms;
-        return ItemPlan{true, (int)std::min<long long>(fp64 ? kShortRows - 1 : kShortRows, std::max(1LL, rows))};
-    }
+    if (!s->tile_probe && strip_rows * 10 <= 41LL * s->sms * kShortRows) return ItemPlan{true, short_rows(s, fp64)};
     const long long wave = (long long)stage_blocks_per_sm(s->precision) * s->sms * kChunk;
     const long long chunks = (strip_rows * 10 + 26 * wave - 1) / (26 * wave);
     return ItemPlan{false, (int)std::min<long long>(s->seg / kChunk, std::max(1LL, chunks)) * kChunk};
@@ -441,7 +460,9 @@ int rebuild(eulbfs_solver* s) {
         }
     }
     const auto taller = [](const int4& a, const int4& b) { return a.w - a.z > b.w - b.z; };
-    std::stable_sort(items.begin(), items.end(), taller);
+    // (short items are of one height within a row, and stay in row order: the
+    // next stage's first items then wait for items claimed long before)
+    if (!plan.short_items) std::stable_sort(items.begin(), items.end(), taller);
     // launches per stage (split domains exchange halos between stages, or
     // eulbfs_set_whole_step(0)): the end of the list in shorter items --
     // kTailLevels times, the last wave (one item per resident CTA) is cut in

@@ -216,6 +216,13 @@ __device__ __forceinline__ R wall_wetting(const Consts<R>& K, const R* in, int s
     return K.four_over_xi * c;
 }
 
+// Phase field of ghost layer k of `side` from the mirror cell's.
+template <class R>
+__device__ __forceinline__ R ghost_C(const Consts<R>& K, int side, int k, R wet, R C) {
+    if (K.bc_c[side] == BC_WETTING || K.bc_c[side] == BC_WETTING_HYST) return C + R(2 * k - 1) * wet * C * (R(1) - C);
+    return C;
+}
+
 // Ghost layer k of `side` from the mirror cell's values; wet = the side's
 // wetting coefficient at this wall position (wall_wetting).
 template <class R>
@@ -227,8 +234,7 @@ __device__ __forceinline__ void apply_ghost(const Consts<R>& K, int side, int k,
     R& ut = x_normal ? q.v : q.u;
     if (f == BC_NOSLIP) { un = -un; ut = -ut; }
     else if (f == BC_SYMMETRY) { un = -un; }
-    if (K.bc_c[side] == BC_WETTING || K.bc_c[side] == BC_WETTING_HYST)
-        q.C = q.C + R(2 * k - 1) * wet * q.C * (R(1) - q.C);
+    q.C = ghost_C(K, side, k, wet, q.C);
 }
 
 template <class R>

@@ -167,7 +167,7 @@ constexpr int kStageThreads = 32 * kChunk;
 // The kernel for short work items (stage_short.cu): at most kShortRows rows,
 // which with their halo fit the 16-row ring at once.
 constexpr int kShortRows = 8;
-constexpr int kShortThreads = 512;
+constexpr int kShortRows64 = 7;   // FP64
 
 // The stage kernel's input tiles: kChunk rows x kTileX columns x all state
 // planes of one buffer, copied into shared memory by a TMA tensor copy.  The

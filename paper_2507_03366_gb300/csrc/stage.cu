@@ -275,7 +275,8 @@ __device__ __forceinline__ void load_rows_tile_muc(Smem<R>& S, int x0, int r0, b
             return k >= 0 ? t[5 * PS + ti] + t[6 * PS + ti] : RC[slot(r0 + k) * RW + cc + d].y;
         };
         S.P.pm[slot(r0 + m)][cc].y =
-            chem_potential_of<R, AXI>(K, Cat(m, 0), Cat(m, 1), Cat(m, -1), Cat(m + 1, 0), Cat(m - 1, 0), x0 + cc - kHalo);
+            chem_potential_of<R, AXI>(K, Cat(m, 0), Cat(m, 1), Cat(m, -1), Cat(m + 1, 0), Cat(m - 1, 0), x0 + cc - kHalo,
+                                     AXI ? S.inv_rc[cc] : R(0));
     }
 }
 
@@ -295,6 +296,7 @@ __device__ __forceinline__ bool sweep_item(Smem<R>& S, const StageLaunch& a, con
     const R ir_f = (AXI && x0 + lane > 0) ? wdiv(R(1), (R)(x0 + lane)) : R(0);
 
     // prologue: rows y0-3 .. y0+2, mu_c of rows y0-2 .. y0+1, y-face row y0
+    column_radii<R, AXI>(S, x0);
     bool ok = true;
     if (tile_rows(S.K, x0, y0 - kHalo, 2 * kHalo)) {
         if (!S.pre) tile_fetch(S, a, stage, x0, y0 - kHalo);   // else copied during the previous item

@@ -50,7 +50,15 @@ struct Core {
     P2<R> YF[3][RING][32];
     P2<R> XF[3][kChunk][32];
     Consts<R> K;
+    R inv_rc[RW];    // axisymmetric domains: 1 / r of the ring columns' cells
 };
+
+// 1 / r of the strip's ring columns (used by mu_c; every CTA thread calls it
+// before the barrier that ends the item's first load phase).
+template <class R, bool AXI>
+__device__ __forceinline__ void column_radii(Core<R>& S, int x0) {
+    if (AXI && threadIdx.x < RW) S.inv_rc[threadIdx.x] = wdiv(R(1), (R)(x0 + (int)threadIdx.x - kHalo) + R(0.5));
+}
 
 __device__ __forceinline__ int slot(int r) { return r & (RING - 1); }
 
@@ -139,11 +147,11 @@ __device__ __forceinline__ void load_rows(Core<R>& S, const R* in, int x0, int r
 // is the 5-point one, or in an axisymmetric domain the conservative
 // (1/r) d/dr (r dC/dr) + d2C/dz2 with faces at r = gx and gx + 1.
 template <class R, bool AXI>
-__device__ __forceinline__ R chem_potential_of(const Consts<R>& K, R c, R ce, R cw, R cn, R cs, int gx) {
+__device__ __forceinline__ R chem_potential_of(const Consts<R>& K, R c, R ce, R cw, R cn, R cs, int gx, R inv_rc) {
     R lap;
     if (AXI) {
         const R rw = (R)gx, re = rw + R(1);
-        lap = wdiv(re * (ce - c) - rw * (c - cw), rw + R(0.5)) + (cn + cs - R(2) * c);
+        lap = fma(re * (ce - c) - rw * (c - cw), inv_rc, cn + cs - R(2) * c);
     } else {
         lap = ce + cw + cn + cs - R(4) * c;
     }
@@ -152,8 +160,10 @@ __device__ __forceinline__ R chem_potential_of(const Consts<R>& K, R c, R ce, R 
 }
 
 template <class R, bool AXI>
-__device__ __forceinline__ R chem_potential(const Consts<R>& K, const P2<R>* RC, int s0, int sN, int sS, int gx) {
-    return chem_potential_of<R, AXI>(K, RC[s0].y, RC[s0 + 1].y, RC[s0 - 1].y, RC[sN].y, RC[sS].y, gx);
+__device__ __forceinline__ R chem_potential(const Core<R>& S, int cc, int sc, int sN, int sS, int x0) {
+    const P2<R>* RC = &S.P.rc[0][0];
+    return chem_potential_of<R, AXI>(S.K, RC[sc].y, RC[sc + 1].y, RC[sc - 1].y, RC[sN].y, RC[sS].y, x0 + cc - kHalo,
+                                     AXI ? S.inv_rc[cc] : R(0));
 }
 
 // True if mu_c of rows [r0, r0 + nrows) of the strip involves no wall ghost
@@ -173,7 +183,6 @@ __device__ __forceinline__ void muc_rows(Core<R>& S, int x0, int r0, int nrows) 
     const Consts<R>& K = S.K;
     constexpr int NC = RW - 2;
     const int total = nrows * NC;
-    const P2<R>* C = &S.P.rc[0][0];
     // a slab's halo rows take mu_c in place, except the outermost (never read)
     const int rlo = K.hlo ? 1 - K.hlo : 0, rhi = K.hhi ? K.ny + K.hhi - 1 : K.ny;
     if ((K.per_x || (x0 >= kHalo - 1 && x0 + NC - (kHalo - 1) <= K.nx)) &&
@@ -184,7 +193,7 @@ __device__ __forceinline__ void muc_rows(Core<R>& S, int x0, int r0, int nrows) 
             const int gy = r0 + rr;
             const int s0 = slot(gy) * RW + cc;
             S.P.pm[slot(gy)][cc].y =
-                chem_potential<R, AXI>(K, C, s0, slot(gy + 1) * RW + cc, slot(gy - 1) * RW + cc, x0 + cc - kHalo);
+                chem_potential<R, AXI>(S, cc, s0, slot(gy + 1) * RW + cc, slot(gy - 1) * RW + cc, x0);
         }
         return;
     }
@@ -206,8 +215,7 @@ __device__ __forceinline__ void muc_rows(Core<R>& S, int x0, int r0, int nrows) 
         }
         R mu = R(0);
         if (!deep)
-            mu = chem_potential<R, AXI>(K, C, slot(my) * RW + mc, slot(my + 1) * RW + mc, slot(my - 1) * RW + mc,
-                                x0 + mc - kHalo);
+            mu = chem_potential<R, AXI>(S, mc, slot(my) * RW + mc, slot(my + 1) * RW + mc, slot(my - 1) * RW + mc, x0);
         S.P.pm[slot(gy)][cc].y = mu;
     }
 }
@@ -468,8 +476,7 @@ __device__ __forceinline__ void recn2(const P2<R>* f, const FaceIdx& x, RecN<R>&
 }
 
 // q at the centre of a side column (e_n = SN, e_t = 0) and at its t-points
-// (e_t = +1: value - d, e_t = -1: value + d), with e.u at the t-points; the
-// forms of side_sums above.
+// (e_t = +1: value - d, e_t = -1: value + d), with e.u at the t-points.
 template <class R, int SN>
 __device__ __forceinline__ R q_centre(R un, R ut) {
     return fma(un, un, fma(R(-0.5) * ut, ut, SN > 0 ? un : -un));
@@ -500,7 +507,7 @@ template <class R, int SN>
 __device__ __forceinline__ R col_dt(const RecN<R>& z) { return SN > 0 ? z.dtl : z.dtr; }
 
 // f (points at dt_f): rho q and q of one side column; sums and differences
-// over the t-points as in side_sums.
+// over its two t-points (e_t = +1 plus / minus -1).
 template <class R>
 struct ColF { R f0, q0, fs, fd, qs, qd; };
 

@@ -24,16 +24,20 @@ namespace eulbfs {
 
 namespace {
 
-constexpr int NTS = kShortThreads;   // 16 warps
-constexpr int NWS = NTS / 32;
+// FP32C: 16 warps.  FP64: 8, so that two CTAs share an SM and one's loads, waits
+// and short phases pass under the other's arithmetic (the FP64 pipe takes 64
+// clocks per warp instruction and sub-core: 8 warps keep it fed).
+template <class R> struct Short;
+template <> struct Short<float> { static constexpr int rows = kShortRows, threads = 512; };
+template <> struct Short<double> { static constexpr int rows = kShortRows64, threads = 256; };
 constexpr int kShortDeps = 64;       // neighbours kept in shared memory (9 one-row items of 3 or 4 strips fit)
 
 template <class R>
 struct ShortSmem : Core<R> {
     // the cell update's inputs: W^n and the stage input by plane, F_s^{n-1} or dF_s/dt
-    R wn[Prec<R>::NP][kShortRows][32];
-    R ws[Prec<R>::NP][kShortRows][32];
-    R frac[kShortRows][32];
+    R wn[Prec<R>::NP][Short<R>::rows][32];
+    R ws[Prec<R>::NP][Short<R>::rows][32];
+    R frac[Short<R>::rows][32];
     // the CTA's next work item, put here by the control warp while the
     // current one runs: its place in the launch, and what it waits for
     int4 item;
@@ -93,17 +97,17 @@ __device__ __forceinline__ void add_release(int* p, int v) {
     asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-__device__ __forceinline__ void put_cell(float (*p)[kShortRows][32], int r, int l, const SV<float>& w) {
+__device__ __forceinline__ void put_cell(float (*p)[Short<float>::rows][32], int r, int l, const SV<float>& w) {
     p[0][r][l] = w.Hh; p[1][r][l] = w.Hl; p[2][r][l] = w.p; p[3][r][l] = w.mx; p[4][r][l] = w.my;
     p[5][r][l] = w.Ch; p[6][r][l] = w.Cl;
 }
-__device__ __forceinline__ void put_cell(double (*p)[kShortRows][32], int r, int l, const SV<double>& w) {
+__device__ __forceinline__ void put_cell(double (*p)[Short<double>::rows][32], int r, int l, const SV<double>& w) {
     p[0][r][l] = w.Hh; p[1][r][l] = w.p; p[2][r][l] = w.mx; p[3][r][l] = w.my; p[4][r][l] = w.Ch;
 }
-__device__ __forceinline__ SV<float> get_cell(const float (*p)[kShortRows][32], int r, int l) {
+__device__ __forceinline__ SV<float> get_cell(const float (*p)[Short<float>::rows][32], int r, int l) {
     return SV<float>{p[0][r][l], p[1][r][l], p[2][r][l], p[3][r][l], p[4][r][l], p[5][r][l], p[6][r][l]};
 }
-__device__ __forceinline__ SV<double> get_cell(const double (*p)[kShortRows][32], int r, int l) {
+__device__ __forceinline__ SV<double> get_cell(const double (*p)[Short<double>::rows][32], int r, int l) {
     return SV<double>{p[0][r][l], 0.0, p[1][r][l], p[2][r][l], p[3][r][l], p[4][r][l], 0.0};
 }
 
@@ -118,9 +122,11 @@ struct SharedCell {
 };
 
 // Load and derive cell (gx, gy) into ring column cc; a halo cell outside the
-// domain is mapped through the boundary rules (as load_rows).
+// domain is mapped through the boundary rules (as load_rows).  Of the outer
+// rows (the third halo row on both sides) only C is ever read, by mu_c.
 template <class R>
-__device__ __forceinline__ SV<R> ring_cell(ShortSmem<R>& S, const R* in, int gx, int gy, int cc, bool inside) {
+__device__ __forceinline__ SV<R> ring_cell(ShortSmem<R>& S, const R* in, int gx, int gy, int cc, bool inside,
+                                           bool outer) {
     const Consts<R>& K = S.K;
     int sx = gx, sy = gy, kx = 0, ky = 0, sdx = XLO, sdy = YLO;
     if (!inside) {
@@ -128,6 +134,13 @@ __device__ __forceinline__ SV<R> ring_cell(ShortSmem<R>& S, const R* in, int gx,
         map_row(K, gy, sy, ky, sdy);
     }
     const SV<R> w = load_state(in, K.plane, (long long)sy * K.nx + sx + K.off);
+    if (outer) {
+        R C = w.Ch + w.Cl;
+        if (kx) C = ghost_C(K, sdx, kx, wall_wetting(K, in, sdx, sy), C);
+        if (ky) C = ghost_C(K, sdy, ky, wall_wetting(K, in, sdy, gx), C);
+        S.P.rc[slot(gy)][cc].y = C;
+        return w;
+    }
     Prim<R> q = derive(K, w);
     if (!inside) {
         // x sides first, then y (corners)
@@ -143,11 +156,13 @@ __device__ __forceinline__ SV<R> ring_cell(ShortSmem<R>& S, const R* in, int gx,
 template <class R, bool AXI, bool GEN>
 __device__ __forceinline__ void short_item(ShortSmem<R>& S, const StageLaunch& a, const int stage, int x0, int y0,
                                            int y1, int claim) {
+    constexpr int NTS = Short<R>::threads, NWS = NTS / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const Consts<R>& K = S.K;
     const R* in = reinterpret_cast<const R*>(K.st[stage]);
     const int rows = y1 - y0;
 
+    column_radii<R, AXI>(S, x0);
     // all loads of the item in one go: the update's inputs of cell (ur, ul) ...
     const int ur = tid / kStripX, ul = tid - ur * kStripX;
     const bool upd = ur < rows && x0 + ul < K.nx;
@@ -163,7 +178,8 @@ __device__ __forceinline__ void short_item(ShortSmem<R>& S, const StageLaunch& a
     const int total = (rows + 2 * kHalo) * RW;
     for (int idx = tid; idx < total; idx += NTS) {
         const int rr = idx / RW, cc = idx - rr * RW;
-        const SV<R> w = ring_cell(S, in, x0 + cc - kHalo, y0 + rr - kHalo, cc, inside);
+        const SV<R> w = ring_cell(S, in, x0 + cc - kHalo, y0 + rr - kHalo, cc, inside,
+                                  rr == 0 || rr == rows + 2 * kHalo - 1);
         const int ir = rr - kHalo, ic = cc - kHalo;
         if (ir >= 0 && ir < rows && ic >= 0 && ic < kStripX) put_cell(S.ws, ir, ic, w);
     }
@@ -204,7 +220,8 @@ __device__ __forceinline__ void short_item(ShortSmem<R>& S, const StageLaunch& a
 }  // namespace
 
 template <class R>
-__global__ void __launch_bounds__(NTS, sizeof(R) == 4 ? 2 : 1) short_kernel(StageLaunch a) {
+__global__ void __launch_bounds__(Short<R>::threads, 2) short_kernel(StageLaunch a) {
+    constexpr int NTS = Short<R>::threads, NWS = NTS / 32;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ShortSmem<R>& S = *reinterpret_cast<ShortSmem<R>*>(smem_raw);
     const int tid = threadIdx.x;
@@ -288,7 +305,7 @@ template <class R>
 cudaError_t launch_t(const StageLaunch& a, int grid, cudaStream_t s) {
     cudaError_t e = configure_t<R>();
     if (e != cudaSuccess) return e;
-    short_kernel<R><<<grid, NTS, sizeof(ShortSmem<R>), s>>>(a);
+    short_kernel<R><<<grid, Short<R>::threads, sizeof(ShortSmem<R>), s>>>(a);
     return cudaGetLastError();
 }
 
@@ -296,7 +313,7 @@ template <class R>
 int blocks_per_sm_t() {
     if (configure_t<R>() != cudaSuccess) return 1;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, short_kernel<R>, NTS, sizeof(ShortSmem<R>)) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, short_kernel<R>, Short<R>::threads, sizeof(ShortSmem<R>)) != cudaSuccess)
         return 1;
     return nb > 0 ? nb : 1;
 }
