@@ -159,6 +159,14 @@ def peak_fma(kind: int, iters: int, stream: Optional[int] = None) -> dict:
     return {"flops_per_s": fl.value, "ms": ms.value, "fma_warp_inst_per_s": wi.value}
 
 
+# A bytes object of a given length with unset contents, and the address of its
+# contents: C may fill a bytes object that nothing else refers to yet.
+_new_bytes = ct.pythonapi.PyBytes_FromStringAndSize
+_new_bytes.restype, _new_bytes.argtypes = ct.py_object, [ct.c_char_p, ct.c_ssize_t]
+_bytes_at = ct.pythonapi.PyBytes_AsString
+_bytes_at.restype, _bytes_at.argtypes = ct.c_void_p, [ct.py_object]
+
+
 def _check(rc: int):
     if rc != OK:
         raise EulbfsError(rc, lib().eulbfs_last_error().decode())
@@ -334,10 +342,10 @@ class Solver:
     def save(self, slot: int = 0):
         """Bitwise-exact checkpoint: (bytes, step)."""
         n = lib().eulbfs_checkpoint_bytes(self._h, slot)
-        buf = ct.create_string_buffer(n)
+        blob = _new_bytes(None, n)           # written in place: no zeroing, no second copy
         step = ct.c_longlong()
-        _check(lib().eulbfs_save(self._h, slot, buf, n, ct.byref(step)))
-        return buf.raw, step.value
+        _check(lib().eulbfs_save(self._h, slot, _bytes_at(blob), n, ct.byref(step)))
+        return blob, step.value
 
     def load(self, blob: bytes, step: int, slot: int = 0):
         _check(lib().eulbfs_load(self._h, slot, blob, len(blob), step))
