@@ -567,7 +567,7 @@ int rebuild(eulbfs_solver* s) {
 }
 
 cudaError_t launch_items(const eulbfs_solver* s, const StageLaunch& a) {
-    return s->short_items ? launch_short(s->precision, a, s->grid, s->stream)
+    return s->short_items ? launch_short(s->precision, a, s->grid, s->grid <= s->sms, s->stream)
                           : launch_stage(s->precision, a, s->grid, s->stream);
 }
 

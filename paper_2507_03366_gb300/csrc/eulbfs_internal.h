@@ -202,7 +202,7 @@ cudaError_t launch_stage(int precision, const StageLaunch& a, int grid, cudaStre
 int stage_blocks_per_sm(int precision);
 size_t stage_smem_bytes(int precision);
 // The same for work items of at most kShortRows rows (any row boundaries).
-cudaError_t launch_short(int precision, const StageLaunch& a, int grid, cudaStream_t s);
+cudaError_t launch_short(int precision, const StageLaunch& a, int grid, bool one_per_sm, cudaStream_t s);
 int short_blocks_per_sm(int precision);
 
 // Initial state from primitive fields (device double arrays); *bad is set

@@ -28,8 +28,10 @@ namespace {
 // and short phases pass under the other's arithmetic (the FP64 pipe takes 64
 // clocks per warp instruction and sub-core: 8 warps keep it fed).
 template <class R> struct Short;
-template <> struct Short<float> { static constexpr int rows = kShortRows, threads = 512; };
-template <> struct Short<double> { static constexpr int rows = kShortRows64, threads = 256; };
+template <> struct Short<float> { static constexpr int rows = kShortRows; };
+template <> struct Short<double> { static constexpr int rows = kShortRows64; };
+template <class R, int PER_SM>
+constexpr int kThreads = sizeof(R) == 8 && PER_SM == 2 ? 256 : 512;
 constexpr int kShortDeps = 64;       // neighbours kept in shared memory (9 one-row items of 3 or 4 strips fit)
 
 template <class R>
@@ -153,10 +155,10 @@ __device__ __forceinline__ SV<R> ring_cell(ShortSmem<R>& S, const R* in, int gx,
 
 // One work item: rows [y0, y1) (at most kShortRows) of the strip at x0.
 // `claim`: the control warp's claimed next position, looked up in here.
-template <class R, bool AXI, bool GEN>
+template <class R, bool AXI, bool GEN, int NTS>
 __device__ __forceinline__ void short_item(ShortSmem<R>& S, const StageLaunch& a, const int stage, int x0, int y0,
                                            int y1, int claim) {
-    constexpr int NTS = Short<R>::threads, NWS = NTS / 32;
+    constexpr int NWS = NTS / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const Consts<R>& K = S.K;
     const R* in = reinterpret_cast<const R*>(K.st[stage]);
@@ -219,9 +221,11 @@ __device__ __forceinline__ void short_item(ShortSmem<R>& S, const StageLaunch& a
 
 }  // namespace
 
-template <class R>
-__global__ void __launch_bounds__(Short<R>::threads, 2) short_kernel(StageLaunch a) {
-    constexpr int NTS = Short<R>::threads, NWS = NTS / 32;
+// PER_SM: resident CTAs per SM.  1 is for batches of at most one item per SM:
+// twice the registers, so nothing spills and more loads are in flight.
+template <class R, int PER_SM>
+__global__ void __launch_bounds__(kThreads<R, PER_SM>, PER_SM) short_kernel(StageLaunch a) {
+    constexpr int NTS = kThreads<R, PER_SM>, NWS = NTS / 32;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ShortSmem<R>& S = *reinterpret_cast<ShortSmem<R>*>(smem_raw);
     const int tid = threadIdx.x;
@@ -264,11 +268,11 @@ __global__ void __launch_bounds__(Short<R>::threads, 2) short_kernel(StageLaunch
         const int x0 = item.y * kStripX;
         const int stage = st % 3;
         if (S.K.gen) {
-            if (S.K.axi) short_item<R, true, true>(S, a, stage, x0, item.z, item.w, claim);
-            else short_item<R, false, true>(S, a, stage, x0, item.z, item.w, claim);
+            if (S.K.axi) short_item<R, true, true, NTS>(S, a, stage, x0, item.z, item.w, claim);
+            else short_item<R, false, true, NTS>(S, a, stage, x0, item.z, item.w, claim);
         } else {
-            if (S.K.axi) short_item<R, true, false>(S, a, stage, x0, item.z, item.w, claim);
-            else short_item<R, false, false>(S, a, stage, x0, item.z, item.w, claim);
+            if (S.K.axi) short_item<R, true, false, NTS>(S, a, stage, x0, item.z, item.w, claim);
+            else short_item<R, false, false, NTS>(S, a, stage, x0, item.z, item.w, claim);
         }
         const int rows = item.w - item.z;
         if (a.stages > 1 && warp < rows && !a.dep_probe) {
@@ -283,7 +287,7 @@ namespace {
 constexpr int kMaxAttrDevices = 64;
 
 // The dynamic shared-memory limit is a per-device attribute (see stage.cu).
-template <class R>
+template <class R, int PER_SM>
 cudaError_t configure_t() {
     static std::mutex m;
     static bool done[kMaxAttrDevices] = {};
@@ -293,7 +297,7 @@ cudaError_t configure_t() {
     if (dev < 0 || dev >= kMaxAttrDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(m);
     if (!done[dev]) {
-        e = cudaFuncSetAttribute(short_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(short_kernel<R, PER_SM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(ShortSmem<R>));
         if (e != cudaSuccess) return e;
         done[dev] = true;
@@ -301,27 +305,28 @@ cudaError_t configure_t() {
     return cudaSuccess;
 }
 
-template <class R>
+template <class R, int PER_SM>
 cudaError_t launch_t(const StageLaunch& a, int grid, cudaStream_t s) {
-    cudaError_t e = configure_t<R>();
+    cudaError_t e = configure_t<R, PER_SM>();
     if (e != cudaSuccess) return e;
-    short_kernel<R><<<grid, Short<R>::threads, sizeof(ShortSmem<R>), s>>>(a);
+    short_kernel<R, PER_SM><<<grid, kThreads<R, PER_SM>, sizeof(ShortSmem<R>), s>>>(a);
     return cudaGetLastError();
 }
 
 template <class R>
 int blocks_per_sm_t() {
-    if (configure_t<R>() != cudaSuccess) return 1;
+    if (configure_t<R, 2>() != cudaSuccess) return 1;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, short_kernel<R>, Short<R>::threads, sizeof(ShortSmem<R>)) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, short_kernel<R, 2>, kThreads<R, 2>, sizeof(ShortSmem<R>)) != cudaSuccess)
         return 1;
     return nb > 0 ? nb : 1;
 }
 
 }  // namespace
 
-cudaError_t launch_short(int precision, const StageLaunch& a, int grid, cudaStream_t s) {
-    return precision == 0 ? launch_t<double>(a, grid, s) : launch_t<float>(a, grid, s);
+cudaError_t launch_short(int precision, const StageLaunch& a, int grid, bool one_per_sm, cudaStream_t s) {
+    if (one_per_sm) return precision == 0 ? launch_t<double, 1>(a, grid, s) : launch_t<float, 1>(a, grid, s);
+    return precision == 0 ? launch_t<double, 2>(a, grid, s) : launch_t<float, 2>(a, grid, s);
 }
 
 int short_blocks_per_sm(int precision) { return precision == 0 ? blocks_per_sm_t<double>() : blocks_per_sm_t<float>(); }
