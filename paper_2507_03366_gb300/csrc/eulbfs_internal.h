@@ -68,10 +68,9 @@ struct Consts {
     //  - the heat capacities of Eq. 6's branches, C_p^sol = x + C~ y and
     //    C_p^liq = z + C~ w: R1 {cp_g, cp_s - cp_g, cp_g, cp_l - cp_g}, as
     //    printed {cp_s, 0, cp_g, cp_l - cp_g};
-    //  - face {Q, C_ref / 6, 6 / C_ref, tau_g - 1/2}; cell {kv, g_x, g_y, 1 / dt}
+    //  - face {3 Q, 3 Q / 4, C_ref / 6, 6 / C_ref}; cell {kv, g_x, g_y, 1 / dt}
     //    and {2 beta, kappa, dt, dt_f}
-    //  - faces with dt_s = 0.5: {3 Q, 3 Q / 4, C_ref / 6, 6 / C_ref}
-    Q4<R> mcp, mrho, mlam, mmu, enth, enthc, facec, cellc, cellc2, facek;
+    Q4<R> mcp, mrho, mlam, mmu, enth, enthc, facek, cellc, cellc2;
     alignas(2 * sizeof(R)) R facet[2];   // (1 - t, t / 6) of t = tau_g - 1/2
     // H_l = C_p^liq hl[0] + hl[1]: R1 {T_l, L}, as printed {0, cp_l T_l + L}
     alignas(2 * sizeof(R)) R hl[2];
@@ -125,7 +124,6 @@ __host__ __device__ inline void fill_consts(const DomainDesc& d, Consts<R>& K) {
     K.hl[0] = printed ? R(0) : (R)d.Tl;
     K.hl[1] = printed ? (R)(d.cp[1] * d.Tl + d.L) : (R)d.L;
     K.printed = printed ? R(1) : R(0);
-    K.facec = make_q4<R>(d.Qg, d.Cref / 6.0, 6.0 / d.Cref, d.tau_g - 0.5);
     K.cellc = make_q4<R>(d.kv, d.gx, d.gy, 1.0 / d.dt);
     K.cellc2 = make_q4<R>(2.0 * d.beta, d.kappa, d.dt, d.dts[1]);
     K.facek = make_q4<R>(3.0 * d.Qg, 0.75 * d.Qg, d.Cref / 6.0, 6.0 / d.Cref);

@@ -242,11 +242,6 @@ __device__ __forceinline__ R face_value8(R l, R r, R ll, R rr) {
 }
 
 template <class R>
-__device__ __forceinline__ R face_value(R l, R r, R ll, R rr) {
-    return R(0.625) * (l + r) - R(0.125) * (ll + rr);
-}
-
-template <class R>
 __device__ __forceinline__ Rec<R> rec_of(R l, R r, R ll, R rr, R lp, R lm, R rp, R rm) {
     Rec<R> z;
     z.l = l;
@@ -266,15 +261,8 @@ __device__ __forceinline__ void rec2(const P2<R>* f, const FaceIdx& x, Rec<R>& a
     b = rec_of(l.y, r.y, ll.y, rr.y, lp.y, lm.y, rp.y, rm.y);
 }
 
-// Face values of both fields of a pair (cells L, R and their outer n-neighbours).
-template <class R>
-__device__ __forceinline__ void face_value2(const P2<R>* f, const FaceIdx& x, R& a, R& b) {
-    const P2<R> l = f[x.L], r = f[x.R], ll = f[x.LL], rr = f[x.RR];
-    a = face_value(l.x, r.x, ll.x, rr.x);
-    b = face_value(l.y, r.y, ll.y, rr.y);
-}
-
-// The same times eight.
+// Eight times the face values of both fields of a pair (cells L, R and their outer
+// n-neighbours).
 template <class R>
 __device__ __forceinline__ void face_value8_2(const P2<R>* f, const FaceIdx& x, R& a, R& b) {
     const P2<R> l = f[x.L], r = f[x.R], ll = f[x.LL], rr = f[x.RR];
@@ -352,6 +340,38 @@ __device__ __forceinline__ SideTerms<R> side_terms(R un, R ut, R rho, R C, R T, 
 // w_a over dt_s.  Of the fluxes only the normal momentum flux changes, by
 // cs^2 dt_s (-rho_f cs^2 u_r / r) = -rho_f u_r / (18 r) with the face values;
 // inv_r = 1 / r of the face (0 on the axis, where the face area is zero).
+//
+// The moments of the surrounding equilibria, scaled as above: 18 sum e_n f, 18 sum
+// e_t f, 18 p_f, C_f, 6 sum e_n g; T_L - T_R and 6 x the rest of sum e_n h; and of
+// f^eq-m the sum of V and the difference of hd of the two sides, p_L + p_R and
+// 8 dt_f (dp_R - dp_L) / 2.
+template <class R>
+struct Moments { R mn, mt, pf, Cf, gn, dT, hn, V, hd, ps, dp; };
+
+// From the moments to the fluxes; Cref6 = C_ref / 6, rho8, cpT64: 8 x rho and 64 x C_p T of the
+// face, ir = 1 / rho8, th, tf: tau_h - 1/2 and tau_f - 1/2.
+template <class R>
+__device__ __forceinline__ FaceFlux<R> close_flux(const Consts<R>& K, const Moments<R>& m, R Cref6, R rho8, R cpT64, R ir,
+                                                  R th, R tf) {
+    // rho_f cs^2 u_f = sum e f^eq (Eq. 56)
+    const R i43 = fma(R(1.0 / 3.0), ir, ir);              // 4/3 ir (a rounded 4/3 would bias every advective flux by 3e-8 in FP32)
+    const R un = m.mn * i43, ut = m.mt * i43;
+    const R ru = rho8 * un;                               // 8 rho_f u_n
+    FaceFlux<R> F;
+    // h* = (1.5 - tau) h^eq(x_f) + (tau - 0.5) h^eq(x_f - e dt_s) (Eq. 13, 16)
+    const R fh = R(1.0 / 64.0) * (cpT64 * un);
+    F.Fh = fma(th, fma(Cref6, m.dT, fma(R(1.0 / 6.0), m.hn, -fh)), fh);
+    F.Fp = R(1.0 / 18.0) * m.mn;                          // sum e_n f^eq(x_f) = rho_f cs^2 u_n,f
+    // f* = (1.5 - tau_f) f^eq(x_f) + (tau_f - 0.5) f^eq-m (Eq. 35, 37 with R3)
+    const R nn = fma(R(2.25), ru * un, m.pf);             // 54 cs^2 (p_f + rho_f u_n^2)
+    F.Fmn = R(1.0 / 54.0) * fma(tf, fma(R(0.375), rho8 * m.V, R(9) * m.ps) - nn, nn);
+    const R nt = ru * ut;                                 // 24 cs^2 rho_f u_n u_t
+    F.Fmt = R(1.0 / 24.0) * fma(tf, fma(R(1.0 / 6.0), fma(rho8, m.hd, m.dp), -nt), nt);
+    F.Fc = fma(K.facet[0], m.Cf * un, K.facet[1] * m.gn);            // Eq. 44, 46
+    F.un = un;
+    return F;
+}
+
 template <class R, bool AXI, class Src>
 __device__ __forceinline__ FaceFlux<R> face_math(const Consts<R>& K, const Src& src, R inv_r) {
     const Q4<R> fc = ld4(K.facek);   // 3 Q, 3 Q / 4, C_ref / 6, 6 / C_ref
@@ -387,26 +407,10 @@ __device__ __forceinline__ FaceFlux<R> face_math(const Consts<R>& K, const Src& 
     const R Cf = fma(R(1.0 / 6.0), fma(R(-1.0 / 16.0), cc, fma(fc.y, fma(R(4), muc.l + muc.r, -muc.f8), L.G + S.G)),
                      R(0.125) * C.f8);                                                           // C_f
     const R gn = fma(fc.x, muc.l - muc.r, L.G - S.G);                                            // 6 sum e_n g
-    // rho_f cs^2 u_f = sum e f^eq (Eq. 56); tau from the face properties (R9)
     const R ir = wdiv(R(1), rho.f8);
-    const R i43 = fma(R(1.0 / 3.0), ir, ir);              // 4/3 ir (a rounded 4/3 would bias every advective flux by 3e-8 in FP32)
-    const R un = mn * i43, ut = mt * i43;
-    const R th = fc.w * (lam8 * ir);                      // tau_h - 0.5 = lambda / (rho C_ref cs^2 dt_s)
-    const R tf = R(6) * (mu8 * ir);                       // tau_f - 0.5 = mu / (rho cs^2 dt_s)
-    const R ru = rho.f8 * un;                             // 8 rho_f u_n
-    FaceFlux<R> F;
-    // h* = (1.5 - tau) h^eq(x_f) + (tau - 0.5) h^eq(x_f - e dt_s) (Eq. 13, 16)
-    const R fh = R(1.0 / 64.0) * ((cp.f8 * T.f8) * un);
-    F.Fh = fma(th, fma(fc.z, T.l - T.r, fma(R(1.0 / 6.0), L.H - S.H, -fh)), fh);
-    F.Fp = R(1.0 / 18.0) * mn;                            // sum e_n f^eq(x_f) = rho_f cs^2 u_n,f
-    // f* = (1.5 - tau_f) f^eq(x_f) + (tau_f - 0.5) f^eq-m (Eq. 35, 37 with R3)
-    const R nn = fma(R(2.25), ru * un, pf);               // 54 cs^2 (p_f + rho_f u_n^2)
-    F.Fmn = R(1.0 / 54.0) * fma(tf, fma(R(0.375), rho.f8 * (L.V + S.V), R(9) * ps) - nn, nn);
-    const R nt = ru * ut;                                 // 24 cs^2 rho_f u_n u_t
-    const R ns = fma(R(2), p.dtr - p.dtl, rho.f8 * (L.hd - S.hd));   // 144 x f^eq-m's
-    F.Fmt = R(1.0 / 24.0) * fma(tf, fma(R(1.0 / 6.0), ns, -nt), nt);
-    F.Fc = fma(K.facet[0], Cf * un, K.facet[1] * gn);       // Eq. 44, 46
-    F.un = un;
+    const Moments<R> m{mn, mt, pf, Cf, gn, T.l - T.r, L.H - S.H, L.V + S.V, L.hd - S.hd, ps, R(2) * (p.dtr - p.dtl)};
+    // tau - 1/2 from the face properties (R9): lambda / (rho C_ref cs^2 dt_s), mu / (rho cs^2 dt_s)
+    FaceFlux<R> F = close_flux(K, m, fc.z, rho.f8, cp.f8 * T.f8, ir, fc.w * (lam8 * ir), R(6) * (mu8 * ir));
     if (AXI) F.Fmn = fma(R(-1.0 / 1152.0) * rho.f8, src.radial(n.f8, t.f8) * inv_r, F.Fmn);
     return F;
 }
@@ -444,27 +448,19 @@ __device__ __forceinline__ FaceFlux<R> face_flux(const Consts<R>& K, const Ring<
 // cell at distance a = 1/2 - dt from the centre along n and dt along t, so
 // its value is f' -/+ (dt/2) d_t f with f' = f + a g_n (g_n the central
 // n-slope of that cell); the face points move by -/+ (dt/4)(d_t f_L + d_t f_R).
-// The closed forms of the linear parts keep their shape with f' for f and
-// dt/12, dt/36 for the t-moments; the nonlinear sums run once per
-// distribution on its own points, by face columns as in face_flux (the
-// centre of a side column at f', its t-points at f' -/+ (dt/2) d_t f).  Used
-// only when some step differs from 1/2; face_flux above is this with a = 0,
-// dt = 1/2.
+// The linear parts keep their closed forms with f' for f and dt/12, dt/36 in
+// the t-moments, and the side columns the terms of side_terms, each
+// distribution's on its own points.  Used only when some step differs from
+// 1/2; face_math above is this with a = 0, dt = 1/2.
 // ---------------------------------------------------------------------------
+// The pieces of one field: cell values, twice their n-slopes, eight times the
+// face value, and the t-differences.
 template <class R>
-struct RecN { R l, r, gl, gr, o0, dtl, dtr; };
+struct RecN { R l, r, gl, gr, f8, dtl, dtr; };
 
 template <class R>
 __device__ __forceinline__ RecN<R> recn_of(R l, R r, R ll, R rr, R lp, R lm, R rp, R rm) {
-    RecN<R> z;
-    z.l = l;
-    z.r = r;
-    z.gl = R(0.5) * (r - ll);
-    z.gr = R(0.5) * (rr - l);
-    z.o0 = R(0.5) * ((z.l + R(0.5) * z.gl) + (z.r - R(0.5) * z.gr));
-    z.dtl = lp - lm;
-    z.dtr = rp - rm;
-    return z;
+    return RecN<R>{l, r, r - ll, rr - l, face_value8(l, r, ll, rr), lp - lm, rp - rm};
 }
 
 template <class R>
@@ -475,169 +471,131 @@ __device__ __forceinline__ void recn2(const P2<R>* f, const FaceIdx& x, RecN<R>&
     b = recn_of(l.y, r.y, ll.y, rr.y, lp.y, lm.y, rp.y, rm.y);
 }
 
-// q at the centre of a side column (e_n = SN, e_t = 0) and at its t-points
-// (e_t = +1: value - d, e_t = -1: value + d), with e.u at the t-points.
-template <class R, int SN>
-__device__ __forceinline__ R q_centre(R un, R ut) {
-    return fma(un, un, fma(R(-0.5) * ut, ut, SN > 0 ? un : -un));
-}
-
-template <class R, int SN>
-__device__ __forceinline__ void eu_tpoints(R un, R ut, R dun, R dut, R& unp, R& utp, R& unm, R& utm, R& eup, R& eum) {
-    unp = un - dun; unm = un + dun; utp = ut - dut; utm = ut + dut;
-    eup = (SN > 0 ? unp : -unp) + utp;
-    eum = (SN > 0 ? unm : -unm) - utm;
-}
-
-template <class R, int SN>
-__device__ __forceinline__ void q_tpoints(R un, R ut, R dun, R dut, R& qp, R& qm) {
-    R unp, utp, unm, utm, eup, eum;
-    eu_tpoints<R, SN>(un, ut, dun, dut, unp, utp, unm, utm, eup, eum);
-    qp = fma(SN > 0 ? unp : -unp, utp, fma(eup, eup, eup));      // e_n e_t = SN
-    qm = fma(SN > 0 ? -unm : unm, utm, fma(eum, eum, eum));      // e_n e_t = -SN
-}
-
-// The value of one field at the centre of a side column for a streaming step
-// with a = 1/2 - dt: the L cell's f + a g_n, the R cell's f - a g_n.
-template <class R, int SN>
-__device__ __forceinline__ R col_centre(const RecN<R>& z, R a) {
-    return SN > 0 ? fma(a, z.gl, z.l) : fma(-a, z.gr, z.r);
-}
-template <class R, int SN>
-__device__ __forceinline__ R col_dt(const RecN<R>& z) { return SN > 0 ? z.dtl : z.dtr; }
-
-// f (points at dt_f): rho q and q of one side column; sums and differences
-// over its two t-points (e_t = +1 plus / minus -1).
+// One distribution's points: h = (1/2 - dt) / 2 of the normal offset (applied to
+// twice the slopes), b = dt / 2 of the tangential one.
 template <class R>
-struct ColF { R f0, q0, fs, fd, qs, qd; };
+struct Points { R h, b; };
+template <class R>
+__device__ __forceinline__ Points<R> points_of(R dt) { return Points<R>{fma(R(-0.5), dt, R(0.25)), R(0.5) * dt}; }
+
+// The value at the centre of a side column, and its t-points' offset.
+template <class R, int SN>
+__device__ __forceinline__ R centre(const RecN<R>& z, const Points<R>& p) {
+    return SN > 0 ? fma(p.h, z.gl, z.l) : fma(-p.h, z.gr, z.r);
+}
+template <class R, int SN>
+__device__ __forceinline__ R offset(const RecN<R>& z, const Points<R>& p) { return p.b * (SN > 0 ? z.dtl : z.dtr); }
+
+// A, B, hq, hd and V of side_terms at one distribution's points.
+template <class R, int SN>
+struct Quad {
+    R un, ut, sun, dn, dt, A, B;
+    __device__ __forceinline__ Quad(const RecN<R>& Un, const RecN<R>& Ut, const Points<R>& p) {
+        un = centre<R, SN>(Un, p);
+        ut = centre<R, SN>(Ut, p);
+        sun = SN > 0 ? un : -un;
+        dn = offset<R, SN>(Un, p);
+        dt = offset<R, SN>(Ut, p);
+        A = sun - dt;
+        B = SN > 0 ? ut - dn : ut + dn;
+    }
+    __device__ __forceinline__ R hq() const {
+        const R x = fma(dn, ut, un * dt);
+        return fma(B, B, fma(A, A, A)) - (SN > 0 ? x : -x);
+    }
+    __device__ __forceinline__ R hd() const {
+        return fma(SN > 0 ? dn : -dn, dt, fma(sun, ut, fma(R(2), A, R(1)) * B));
+    }
+    __device__ __forceinline__ R V(R hq_) const { return fma(R(2), fma(un, un, fma(R(-0.5) * ut, ut, sun)), hq_); }
+};
+
+template <class R>
+struct ColF { R X, V, hd, F; };
 
 template <class R, int SN>
-__device__ __forceinline__ ColF<R> col_f(const RecN<R>& Un, const RecN<R>& Ut, const RecN<R>& Rho, R a, R b) {
+__device__ __forceinline__ ColF<R> col_f(const RecN<R>& Un, const RecN<R>& Ut, const RecN<R>& Rho, const Points<R>& p) {
+    const Quad<R, SN> q(Un, Ut, p);
+    const R rho = centre<R, SN>(Rho, p), dr = offset<R, SN>(Rho, p), hq = q.hq();
     ColF<R> s;
-    const R un = col_centre<R, SN>(Un, a), ut = col_centre<R, SN>(Ut, a), rho = col_centre<R, SN>(Rho, a);
-    s.q0 = q_centre<R, SN>(un, ut);
-    s.f0 = rho * s.q0;
-    R qp, qm;
-    q_tpoints<R, SN>(un, ut, b * col_dt<R, SN>(Un), b * col_dt<R, SN>(Ut), qp, qm);
-    const R dr = b * col_dt<R, SN>(Rho);
-    const R am = (rho + dr) * qm;
-    s.fs = fma(rho - dr, qp, am);
-    s.fd = fma(rho - dr, qp, -am);
-    s.qs = qp + qm;
-    s.qd = qp - qm;
+    s.hd = q.hd();
+    s.V = q.V(hq);
+    s.X = fma(rho, s.V, -(dr * s.hd));
+    s.F = fma(rho, s.hd, -(dr * hq));
     return s;
 }
 
-// g (points at dt_g): C u_n at the centre and the t-points' sum of C e.u.
 template <class R, int SN>
-__device__ __forceinline__ void col_g(const RecN<R>& Un, const RecN<R>& Ut, const RecN<R>& Cc, R a, R b, R& c0, R& cs) {
-    const R un = col_centre<R, SN>(Un, a), ut = col_centre<R, SN>(Ut, a), C = col_centre<R, SN>(Cc, a);
-    c0 = C * un;
-    R unp, utp, unm, utm, eup, eum;
-    eu_tpoints<R, SN>(un, ut, b * col_dt<R, SN>(Un), b * col_dt<R, SN>(Ut), unp, utp, unm, utm, eup, eum);
-    const R dC = b * col_dt<R, SN>(Cc);
-    cs = fma(C - dC, eup, (C + dC) * eum);
+__device__ __forceinline__ R col_g(const RecN<R>& Un, const RecN<R>& Ut, const RecN<R>& C, const Points<R>& p) {
+    const Quad<R, SN> q(Un, Ut, p);
+    return fma(centre<R, SN>(C, p), fma(R(2), q.sun, q.A), -(offset<R, SN>(C, p) * q.B));
 }
 
-// h (points at dt_h): C_p T q at the centre and the t-points' sum.
 template <class R, int SN>
-__device__ __forceinline__ void col_h(const RecN<R>& Un, const RecN<R>& Ut, const RecN<R>& T, const RecN<R>& cp, R a,
-                                      R b, R& h0, R& hs) {
-    const R un = col_centre<R, SN>(Un, a), ut = col_centre<R, SN>(Ut, a);
-    const R Tc = col_centre<R, SN>(T, a), cc = col_centre<R, SN>(cp, a);
-    h0 = (cc * Tc) * q_centre<R, SN>(un, ut);
-    R qp, qm;
-    q_tpoints<R, SN>(un, ut, b * col_dt<R, SN>(Un), b * col_dt<R, SN>(Ut), qp, qm);
-    const R dT = b * col_dt<R, SN>(T), dc = b * col_dt<R, SN>(cp);
-    hs = fma((cc - dc) * (Tc - dT), qp, ((cc + dc) * (Tc + dT)) * qm);
+__device__ __forceinline__ R col_h(const RecN<R>& Un, const RecN<R>& Ut, const RecN<R>& T, const RecN<R>& cp,
+                                   const Points<R>& p) {
+    const Quad<R, SN> q(Un, Ut, p);
+    const R t = centre<R, SN>(T, p), c = centre<R, SN>(cp, p), dT = offset<R, SN>(T, p), dc = offset<R, SN>(cp, p);
+    const R hq = q.hq();
+    return fma(-fma(dc, t, c * dT), q.hd(), fma(dc * dT, hq, (c * t) * q.V(hq)));
 }
 
 template <class R, bool AXI>
 __device__ __forceinline__ FaceFlux<R> face_flux_gen(const Consts<R>& K, const Ring<R>& P, const FaceIdx& x,
                                                      bool normal_x, bool normal_is_r, R inv_r) {
-    const R w1 = R(1.0 / 9.0), w5 = R(1.0 / 36.0);
+    const Points<R> pf_ = points_of(K.dtf), pg_ = points_of(K.dtg), ph_ = points_of(K.dth);
     RecN<R> Un, Ut;
     recn2(&P.uv[0][0], x, Un, Ut);
     if (!normal_x) { const RecN<R> t = Un; Un = Ut; Ut = t; }
-    RecN<R> Rho, Cc;
-    recn2(&P.rc[0][0], x, Rho, Cc);
-    // f: points at dt_f; the face column (e_n = 0) shifts by (dt/4)(d_t f_L + d_t f_R)
-    R pf_n, mn_n, mt_n, Snn_q, Snt_q;
-    const R rho_f = Rho.o0;
-    {
-        const R a = R(0.5) - K.dtf, b = R(0.5) * K.dtf, h = R(0.5) * b;
-        const ColF<R> L = col_f<R, 1>(Un, Ut, Rho, a, b);
-        const ColF<R> Rs = col_f<R, -1>(Un, Ut, Rho, a, b);
-        const R stn = h * (Un.dtl + Un.dtr), stt = h * (Ut.dtl + Ut.dtr), str = h * (Rho.dtl + Rho.dtr);
-        const R un2 = Un.o0 - stn, un4 = Un.o0 + stn, ut2 = Ut.o0 - stt, ut4 = Ut.o0 + stt;
-        const R q2 = fma(ut2, ut2, fma(R(-0.5) * un2, un2, ut2));
-        const R q4 = fma(ut4, ut4, fma(R(-0.5) * un4, un4, -ut4));
-        const R a4 = (Rho.o0 + str) * q4;
-        const R f24s = fma(Rho.o0 - str, q2, a4), f24d = fma(Rho.o0 - str, q2, -a4);
-        const R ruu0 = rho_f * fma(Un.o0, Un.o0, Ut.o0 * Ut.o0);
-        pf_n = R(-2.0 / 9.0) * ruu0 + w1 * ((L.f0 + Rs.f0) + f24s) + w5 * (L.fs + Rs.fs);
-        mn_n = w1 * (L.f0 - Rs.f0) + w5 * (L.fs - Rs.fs);
-        mt_n = w1 * f24d + w5 * (L.fd + Rs.fd);
-        Snn_q = w1 * (L.q0 + Rs.q0) + w5 * (L.qs + Rs.qs);
-        Snt_q = w5 * (L.qd - Rs.qd);
-    }
-    // g: points at dt_g
-    R ce_a, cen_a, ce_d, cen_d;
-    {
-        const R a = R(0.5) - K.dtg, b = R(0.5) * K.dtg, h = R(0.5) * b;
-        R c0L, csL, c0R, csR;
-        col_g<R, 1>(Un, Ut, Cc, a, b, c0L, csL);
-        col_g<R, -1>(Un, Ut, Cc, a, b, c0R, csR);
-        const R stt = h * (Ut.dtl + Ut.dtr), stc = h * (Cc.dtl + Cc.dtr);
-        const R c24 = fma(Cc.o0 - stc, Ut.o0 - stt, -((Cc.o0 + stc) * (Ut.o0 + stt)));
-        ce_a = (c0L - c0R) + c24;
-        cen_a = c0L + c0R;
-        ce_d = csL + csR;
-        cen_d = csL - csR;
-    }
+    const R Sn = Un.dtl + Un.dtr, St = Ut.dtl + Ut.dtr;
+    Moments<R> m;
     // h: points at dt_h (only e_n != 0 points carry C_p T q into the flux)
     RecN<R> T, cp;
     recn2(&P.tc[0][0], x, T, cp);
-    R th_a, th_d;
+    m.hn = col_h<R, 1>(Un, Ut, T, cp, ph_) - col_h<R, -1>(Un, Ut, T, cp, ph_);
+    m.dT = centre<R, 1>(T, ph_) - centre<R, -1>(T, ph_);
+    RecN<R> Rho, Cc;
+    recn2(&P.rc[0][0], x, Rho, Cc);
+    const R rho8 = Rho.f8;
+    // g: points at dt_g
+    R cf;
     {
-        const R a = R(0.5) - K.dth, b = R(0.5) * K.dth;
-        R h0L, hsL, h0R, hsR;
-        col_h<R, 1>(Un, Ut, T, cp, a, b, h0L, hsL);
-        col_h<R, -1>(Un, Ut, T, cp, a, b, h0R, hsR);
-        th_a = h0L - h0R;
-        th_d = hsL - hsR;
+        const R L = col_g<R, 1>(Un, Ut, Cc, pg_), S = col_g<R, -1>(Un, Ut, Cc, pg_);
+        const R w = R(4) * pg_.b;
+        cf = fma(R(-1.0 / 16.0) * w, fma(Cc.f8, St, (Cc.dtl + Cc.dtr) * Ut.f8), L + S);
+        m.gn = L - S;
+    }
+    // f: points at dt_f; the face column as in face_math, its steps 8 (dt/4)(dt_L + dt_R)
+    {
+        const ColF<R> L = col_f<R, 1>(Un, Ut, Rho, pf_), S = col_f<R, -1>(Un, Ut, Rho, pf_);
+        const R w = R(4) * pf_.b;
+        const R sn = w * Sn, st = w * St, sr = w * (Rho.dtl + Rho.dtr);
+        const R a = Un.f8 * Un.f8, b = Ut.f8 * Ut.f8;
+        const R hs = fma(R(-0.5), fma(sn, sn, a), fma(R(-8), st, fma(st, st, b)));
+        const R hd = fma(Un.f8, sn, fma(R(-2), st, R(8)) * Ut.f8);
+        const R G0 = fma(rho8, hs - (a + b), -(sr * hd)), Gt = fma(rho8, hd, -(sr * hs));
+        m.mn = L.X - S.X;
+        m.pf = fma(R(1.0 / 128.0), G0, L.X + S.X);
+        m.mt = fma(R(1.0 / 128.0), Gt, L.F + S.F);
+        m.V = L.V + S.V;
+        m.hd = L.hd - S.hd;
     }
     RecN<R> p, mu;
     recn2(&P.pm[0][0], x, p, mu);
-    R lamf, muf;
-    face_value2(&P.lm[0][0], x, lamf, muf);
-    const Q4<R> fc = ld4(K.facec);   // Q, C_ref / 6, 6 / C_ref, tau_g - 1/2
-    const R af = R(0.5) - K.dtf, ag = R(0.5) - K.dtg, ah = R(0.5) - K.dth;
-    const R pl = p.l + af * p.gl, pr = p.r - af * p.gr;
-    const R ml = mu.l + ag * mu.gl, mr = mu.r - ag * mu.gr;
-    const R Tl = T.l + ah * T.gl, Tr = T.r - ah * T.gr;
-    const R pf = R(2.0 / 3.0) * p.o0 + R(1.0 / 6.0) * (pl + pr) + pf_n;
-    const R mn = R(1.0 / 6.0) * (pl - pr) + mn_n;
-    const R mt = -(K.dtf * R(1.0 / 12.0)) * (p.dtl + p.dtr) + mt_n;
-    const R Cf = Cc.o0 + fc.x * (R(0.5) * (ml + mr) - mu.o0) + R(1.0 / 3.0) * ce_a + R(1.0 / 12.0) * ce_d;
-    const R Sg = R(0.5) * fc.x * (ml - mr) + R(1.0 / 3.0) * cen_a + R(1.0 / 12.0) * cen_d;
-    const R Sh = fc.y * (Tl - Tr) + R(1.0 / 3.0) * th_a + R(1.0 / 12.0) * th_d;
-    const R Snn_p = R(1.0 / 6.0) * (pl + pr);
-    const R Snt_p = (K.dtf * R(1.0 / 36.0)) * (p.dtr - p.dtl);
-    const R irf = wdiv(R(1), rho_f);
-    const R unf = R(3) * mn * irf, utf = R(3) * mt * irf;
-    const R th = K.th_coef * lamf * irf;
-    const R tf = K.tf_coef * muf * irf;
-    const R tg = fc.w;
-    const R cs2 = R(1.0 / 3.0);
-    FaceFlux<R> F;
-    F.Fh = (R(1) - th) * (cp.o0 * T.o0) * unf + th * Sh;
-    F.Fp = mn;
-    F.Fmn = (R(1) - tf) * cs2 * (pf + rho_f * unf * unf) + tf * (Snn_p + rho_f * Snn_q);
-    F.Fmt = (R(1) - tf) * cs2 * rho_f * unf * utf + tf * (Snt_p + rho_f * Snt_q);
-    F.Fc = (R(1) - tg) * Cf * unf + tg * Sg;
-    F.un = unf;
-    if (AXI) F.Fmn += -(K.dtf * R(1.0 / 9.0)) * rho_f * (normal_is_r ? Un.o0 : Ut.o0) * inv_r;
+    R lam8, mu8;
+    face_value8_2(&P.lm[0][0], x, lam8, mu8);
+    const Q4<R> fc = ld4(K.facek);   // 3 Q, 3 Q / 4, C_ref / 6, 6 / C_ref
+    const R pl = centre<R, 1>(p, pf_), pr = centre<R, -1>(p, pf_);
+    const R ml = centre<R, 1>(mu, pg_), mr = centre<R, -1>(mu, pg_);
+    m.ps = pl + pr;
+    m.mn = fma(R(3), pl - pr, m.mn);
+    m.pf = fma(R(1.5), p.f8, fma(R(3), m.ps, m.pf));
+    m.mt = fma(R(-3) * pf_.b, p.dtl + p.dtr, m.mt);
+    m.dp = (R(8) * pf_.b) * (p.dtr - p.dtl);
+    m.Cf = fma(R(1.0 / 6.0), fma(fc.y, fma(R(4), ml + mr, -mu.f8), cf), R(0.125) * Cc.f8);
+    m.gn = fma(fc.x, ml - mr, m.gn);
+    const R ir = wdiv(R(1), rho8);
+    FaceFlux<R> F = close_flux(K, m, fc.z, rho8, cp.f8 * T.f8, ir, K.th_coef * (lam8 * ir), K.tf_coef * (mu8 * ir));
+    if (AXI) F.Fmn = fma(R(-1.0 / 576.0) * K.dtf * rho8, (normal_is_r ? Un.f8 : Ut.f8) * inv_r, F.Fmn);
     return F;
 }
 
@@ -736,10 +694,9 @@ __device__ __forceinline__ void cell_update(Core<R>& S, const Cell& in, int stag
     const R Fl = (&P.fl[0][0])[q];
     const P2<R>* RC = &P.rc[0][0];
     const P2<R>* PM = &P.pm[0][0];
-    const R drx = R(0.5) * (RC[q + 1].x - RC[q - 1].x);
-    const R dry = R(0.5) * (RC[qn].x - RC[qs].x);
-    const R dmx = R(0.5) * (PM[q + 1].y - PM[q - 1].y);
-    const R dmy = R(0.5) * (PM[qn].y - PM[qs].y);
+    // twice the central slopes of rho and mu_c
+    const R drx = RC[q + 1].x - RC[q - 1].x, dry = RC[qn].x - RC[qs].x;
+    const R dmx = PM[q + 1].y - PM[q - 1].y, dmy = PM[qn].y - PM[qs].y;
     const Q4<R> cc = ld4(K.cellc);   // kv, g_x, g_y, 1 / dt
     R dfs;
     if (stage == 0) {   // reading R14: lagged dF_s/dt, fixed over the step
@@ -751,15 +708,16 @@ __device__ __forceinline__ void cell_update(Core<R>& S, const Cell& in, int stag
         dfs = in.frac();
     }
     const R cs2 = R(1.0 / 3.0);
-    const R D = solid_gate(K, C) * dfs;
-    Rk[0] += Cp * T * divu;                                           // Eq. 51 row 1
-    Rk[1] += u * (drx * cs2) + v * (dry * cs2) + rho * cs2 * cc.x * D;   // row 2
-    Rk[2] += cs2 * (-Fl * C * dmx + rho * cc.y - rho * u * D);         // row 3 (R13)
-    Rk[3] += cs2 * (-Fl * C * dmy + rho * cc.z - rho * v * D);         // row 4
-    Rk[4] += C * cc.x * dfs;                                           // row 5 (R12: Eq. 40 / 47)
+    const R rD = rho * (solid_gate(K, C) * dfs);
+    const R hFC = R(0.5) * (Fl * C);
+    Rk[0] = fma(Cp * T, divu, Rk[0]);                                                       // Eq. 51 row 1
+    Rk[1] = fma(R(1.0 / 6.0), fma(u, drx, v * dry), fma(cs2 * cc.x, rD, Rk[1]));            // row 2
+    Rk[2] = fma(cs2, fma(rho, cc.y, -fma(hFC, dmx, u * rD)), Rk[2]);                        // row 3 (R13)
+    Rk[3] = fma(cs2, fma(rho, cc.z, -fma(hFC, dmy, v * rD)), Rk[3]);                        // row 4
+    Rk[4] = fma(C * cc.x, dfs, Rk[4]);                                                      // row 5 (R12: Eq. 40 / 47)
     const Q4<R> c2 = ld4(K.cellc2);   // dt, dt_f in z, w
     if (AXI)   // hoop stress Pi_thetatheta / r with the pressure advanced over dt_s (reading R24)
-        Rk[2] += cs2 * (PM[q].x - c2.w * divF1 - R(2) * (&P.lm[0][0])[q].y * u * irc) * irc;
+        Rk[2] = fma(cs2 * irc, fma(R(-2) * irc, (&P.lm[0][0])[q].y * u, fma(-c2.w, divF1, PM[q].x)), Rk[2]);
 
     // stage 0 reads W^n as its input: one load serves both
     const SV<R> wn = in.wn();
