@@ -235,6 +235,7 @@ struct eulbfs_solver {
     int graph_steps = 0;
     cudaGraphExec_t graph = nullptr;
     bool graph_valid = false;
+    bool capturing = false;        // launches are being recorded: a graph's own edges are quicker than launch_behind's
     // the last eulbfs_autotune: candidate heights and their best ms per step
     int tune_n = 0;
     int tune_rows[kMaxTune] = {};
@@ -588,6 +589,7 @@ int launch_steps_direct(eulbfs_solver* s, long long k) {
     a.dep_off = s->d_deps;
     a.dep_idx = s->d_deps + (s->nitems + 1);
     a.stage = 0;
+    a.behind = 0;
     static const char* const kStageRange[3] = {"eulbfs RK stage 1", "eulbfs RK stage 2", "eulbfs RK stage 3"};
     while (k > 0) {
         // counters and done flags start at zero every launch: an aborted launch cannot leave one behind
@@ -605,13 +607,15 @@ int launch_steps_direct(eulbfs_solver* s, long long k) {
             a.stages = 1;
             for (int st = 0; st < 3; ++st) {
                 a.stage = st;
+                // the first stage follows the counters' memset
+                a.behind = st > 0 && !s->capturing;
                 nvtxRangePushA(kStageRange[st]);
                 cudaError_t e = launch_items(s, a);
                 ++s->launches;
                 // split domains: the stage's output halos from the neighbouring slabs
                 if (e == cudaSuccess && s->nlinks) {
                     e = launch_halo(s->precision, s->d_consts, s->d_links, s->nlinks, s->link_nx, st == 2 ? 0 : st + 1,
-                                    s->stream);
+                                    !s->capturing, s->stream);
                     ++s->launches;
                 }
                 nvtxRangePop();
@@ -631,7 +635,9 @@ int capture_graph(eulbfs_solver* s) {
     }
     // the capture records launches without running them: count them once per replay
     const unsigned long long before = s->launches;
+    s->capturing = true;
     int rc = launch_steps_direct(s, s->graph_steps);
+    s->capturing = false;
     s->graph_launches = s->launches - before;
     s->launches = before;
     cudaGraph_t g = nullptr;
@@ -1019,7 +1025,7 @@ int eulbfs_step(eulbfs_solver* s, long long n) {
         if (s->nitems == 0) break;
         if (s->halo_stale) {   // W^n written by creation, set_state or load: its halos first
             if (s->nlinks) {
-                CK(launch_halo(s->precision, s->d_consts, s->d_links, s->nlinks, s->link_nx, 0, s->stream), "halo rows");
+                CK(launch_halo(s->precision, s->d_consts, s->d_links, s->nlinks, s->link_nx, 0, false, s->stream), "halo rows");
                 ++s->launches;
             }
             s->halo_stale = false;

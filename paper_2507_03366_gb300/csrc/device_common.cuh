@@ -12,6 +12,11 @@ namespace eulbfs {
 enum { BC_PERIODIC = 0, BC_DIRICHLET_T, BC_ADIABATIC, BC_NOSLIP, BC_SYMMETRY, BC_OUTLET, BC_NOFLUX, BC_WETTING,
        BC_WETTING_HYST };
 
+// Programmatic dependent launch: let the next kernel of the stream start, and
+// wait for the kernels before this one (both do nothing without the attribute).
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 template <class R> struct Prec;
 template <> struct Prec<double> { static constexpr int NP = 5; };
 template <> struct Prec<float> { static constexpr int NP = 7; };

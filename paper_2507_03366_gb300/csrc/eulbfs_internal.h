@@ -189,6 +189,7 @@ struct StageLaunch {
     const int* dep_idx;
     int* done;               // [stages][nitems], zeroed before each launch
     int* flag;               // bit 0: non-finite state seen; bit 1: a bounded wait (tile or neighbour) gave up
+    int behind;              // 1: the kernel before it in the stream lets it start early (launch_behind)
     unsigned tile_probe;     // bytes each tile barrier expects beyond its copy (0; > 0 only to test the bounded waits)
     int dep_probe;           // 1: items never mark themselves done (only to test the bounded neighbour waits)
 };
@@ -196,6 +197,30 @@ struct StageLaunch {
 // Launch one Runge-Kutta stage (stages == 1) or k whole steps (stages == 3 k)
 // over every work item of the batch.
 cudaError_t launch_stage(int precision, const StageLaunch& a, int grid, cudaStream_t s);
+
+// Launch `kernel` so that its CTAs may start while the kernel before it in the
+// stream drains, if that kernel calls launch_dependents(); it has to call
+// wait_prior() before it reads or writes anything the other one touches.
+// For the launches per stage of split domains, whose gaps cost more than their
+// halo copies: us per step with three stages and three copies, 256^2 in four
+// slabs 45.1 -> 36.3, 512^2 in two 90.7 -> 81.5, 768^2 in four 140.7 -> 134.2 (in
+// a captured graph, whose edges are quick by themselves: 34.9, 80.7, 130.4).
+template <class... P, class... A>
+inline cudaError_t launch_behind(bool behind, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                                 A... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = behind ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 // Resident CTAs per SM of the stage kernel (for sizing the persistent grid).
 int stage_blocks_per_sm(int precision);
 size_t stage_smem_bytes(int precision);
@@ -223,7 +248,7 @@ cudaError_t launch_set_state(int precision, const DomainDesc* d_desc, long long 
 // slab's lower halo and the upper slab's bottom kHalo rows to the lower
 // slab's upper halo, in state buffer `buffer` (all planes).
 cudaError_t launch_halo(int precision, const void* consts, const int2* links, int nlinks, int max_nx, int buffer,
-                        cudaStream_t s);
+                        bool behind, cudaStream_t s);
 
 // FP64 diagnostics: per-block partial sums (deterministic order) and the final pass.
 constexpr int kDiagThreads = 256;

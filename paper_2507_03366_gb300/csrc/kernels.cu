@@ -137,6 +137,8 @@ __global__ void set_state_kernel(const DomainDesc* dd, long long n, const double
 // ---------------------------------------------------------------------------
 template <class R>
 __global__ void halo_kernel(const Consts<R>* consts, const int2* links, int buffer) {
+    launch_dependents();
+    wait_prior();
     const int2 lk = links[blockIdx.y];
     const Consts<R>& A = consts[lk.x];
     const Consts<R>& B = consts[lk.y];
@@ -159,15 +161,15 @@ __global__ void halo_kernel(const Consts<R>* consts, const int2* links, int buff
 }
 
 cudaError_t launch_halo(int precision, const void* consts, const int2* links, int nlinks, int max_nx, int buffer,
-                        cudaStream_t s) {
+                        bool behind, cudaStream_t s) {
     if (nlinks <= 0) return cudaSuccess;
     const long long work = 2LL * (precision == 0 ? 5 : 7) * kHalo * max_nx;
     const dim3 grid((unsigned)std::min<long long>((work + 255) / 256, 1024), (unsigned)nlinks);
     if (precision == 0)
-        halo_kernel<double><<<grid, 256, 0, s>>>(static_cast<const Consts<double>*>(consts), links, buffer);
-    else
-        halo_kernel<float><<<grid, 256, 0, s>>>(static_cast<const Consts<float>*>(consts), links, buffer);
-    return cudaGetLastError();
+        return launch_behind(behind, halo_kernel<double>, grid, 256, 0, s, static_cast<const Consts<double>*>(consts), links,
+                             buffer);
+    return launch_behind(behind, halo_kernel<float>, grid, 256, 0, s, static_cast<const Consts<float>*>(consts), links,
+                         buffer);
 }
 
 static int grid_for(long long n) {

@@ -373,6 +373,8 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 4 : 2) stage_kernel(Stage
         bar_init(&S.tile_bar);
     }
     __syncthreads();
+    launch_dependents();
+    wait_prior();
     const Consts<R>* consts = static_cast<const Consts<R>*>(a.consts);
     TileIO io{0u};
 
@@ -463,8 +465,7 @@ template <class R>
 static cudaError_t launch_t(const StageLaunch& a, int grid, cudaStream_t s) {
     cudaError_t e = configure_t<R>();
     if (e != cudaSuccess) return e;
-    stage_kernel<R><<<grid, NT, sizeof(Smem<R>), s>>>(a);
-    return cudaGetLastError();
+    return launch_behind(a.behind, stage_kernel<R>, dim3(grid), NT, sizeof(Smem<R>), s, a);
 }
 
 template <class R>

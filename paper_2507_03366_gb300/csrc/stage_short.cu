@@ -232,6 +232,8 @@ __global__ void __launch_bounds__(kThreads<R, PER_SM>, PER_SM) short_kernel(Stag
     const Consts<R>* consts = static_cast<const Consts<R>*>(a.consts);
     int* const counter = a.work + (a.stages == 1 ? a.stage : 0);
     const int lane = tid & 31, warp = tid >> 5;
+    launch_dependents();
+    wait_prior();
     // items are claimed in order, one ahead, as in stage.cu: every item waits
     // only for items claimed before it
     if (warp == NWS - 1) {
@@ -309,8 +311,7 @@ template <class R, int PER_SM>
 cudaError_t launch_t(const StageLaunch& a, int grid, cudaStream_t s) {
     cudaError_t e = configure_t<R, PER_SM>();
     if (e != cudaSuccess) return e;
-    short_kernel<R, PER_SM><<<grid, kThreads<R, PER_SM>, sizeof(ShortSmem<R>), s>>>(a);
-    return cudaGetLastError();
+    return launch_behind(a.behind, short_kernel<R, PER_SM>, dim3(grid), kThreads<R, PER_SM>, sizeof(ShortSmem<R>), s, a);
 }
 
 template <class R>
