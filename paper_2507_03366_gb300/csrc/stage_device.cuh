@@ -76,29 +76,6 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
     return v;
 }
 
-// Whole-step launches: true once every stage st - 1 item whose output item i
-// of stage st reads is done (acquire loads; the caller's barrier then
-// publishes the data to its CTA).  Lanes of one warp take one neighbour each.
-// A bounded wait: after 2^31 clocks it gives up and returns false.
-__device__ __forceinline__ bool deps_ready(const StageLaunch& a, int st, int i, int lane, bool wait,
-                                           unsigned sleep_ns = 256) {
-    // one-stage launches have no neighbourhood lists (kernel boundaries order the stages)
-    if (a.stages == 1 || st == 0) return true;
-    const int* done = a.done + (size_t)(st - 1) * a.nitems;
-    bool ok = true;
-    for (int j = a.dep_off[i] + lane; j < a.dep_off[i + 1]; j += 32) {
-        const int* f = done + a.dep_idx[j];
-        if (ld_acquire(f)) continue;
-        if (!wait) { ok = false; continue; }
-        const long long t0 = clock64();
-        while (!ld_acquire(f)) {
-            if (clock64() - t0 > (1LL << 31)) { ok = false; break; }
-            if (sleep_ns) __nanosleep(sleep_ns);
-        }
-    }
-    return __all_sync(0xffffffffu, ok);
-}
-
 // Step 1: rows [r0, r0 + nrows) of the strip (all RW columns).
 template <class R>
 __device__ __forceinline__ void store_prim(Core<R>& S, int s, int cc, const Prim<R>& q) {

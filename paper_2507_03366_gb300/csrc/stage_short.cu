@@ -79,8 +79,8 @@ __device__ __forceinline__ void look_up(ShortSmem<R>& S, const StageLaunch& a, i
 
 // Wait until every item that the current one reads has finished the previous
 // stage (one warp; lanes take one neighbour each).  A bounded wait, as
-// deps_ready of stage_device.cuh, but it polls without sleeping: the next
-// stage starts when the slowest neighbour's flag is seen.
+// next_ready of stage.cu, but it polls without sleeping: the next stage
+// starts when the slowest neighbour's flag is seen.
 template <class R>
 __device__ __forceinline__ bool wait_deps(const ShortSmem<R>& S, const StageLaunch& a, int st, int n, int lane) {
     const int* done = a.done + (size_t)(st - 1) * a.nitems;
