@@ -330,7 +330,8 @@ __device__ __forceinline__ void load_rows_tile_muc(Smem<R>& S, int x0, int r0, b
             return k >= 0 ? t[5 * PS + ti] + t[6 * PS + ti] : RC[slot(r0 + k) * RW + cc + d].y;
         };
         S.P.pm[slot(r0 + m)][cc].y =
-            chem_potential_of<R, AXI>(K, Cat(m, 0), Cat(m, 1), Cat(m, -1), Cat(m + 1, 0), Cat(m - 1, 0), x0 + cc - kHalo,
+            chem_potential_of<R, AXI>(K, Cat(m, 0), Cat(m, 1), Cat(m, -1), Cat(m + 1, 0), Cat(m - 1, 0),
+                                     AXI ? left_radius(S, cc, x0 + cc - kHalo) : R(0),
                                      AXI ? S.inv_rc[cc] : R(0));
     }
 }

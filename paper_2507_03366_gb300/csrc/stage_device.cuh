@@ -51,13 +51,22 @@ struct Core {
     P2<R> XF[3][kChunk][32];
     Consts<R> K;
     R inv_rc[RW];    // axisymmetric domains: 1 / r of the ring columns' cells
+    R rw[sizeof(R) == 8 ? RW : 1];   // and the radius of their left faces (FP64: conversions are slow)
 };
+
+// The radius of the left face of ring column cc (column gx of the domain).
+__device__ __forceinline__ float left_radius(const Core<float>&, int, int gx) { return (float)gx; }
+__device__ __forceinline__ double left_radius(const Core<double>& S, int cc, int) { return S.rw[cc]; }
 
 // 1 / r of the strip's ring columns (used by mu_c; every CTA thread calls it
 // before the barrier that ends the item's first load phase).
 template <class R, bool AXI>
 __device__ __forceinline__ void column_radii(Core<R>& S, int x0) {
-    if (AXI && threadIdx.x < RW) S.inv_rc[threadIdx.x] = wdiv(R(1), (R)(x0 + (int)threadIdx.x - kHalo) + R(0.5));
+    if (AXI && threadIdx.x < RW) {
+        const R rw = (R)(x0 + (int)threadIdx.x - kHalo);
+        S.inv_rc[threadIdx.x] = wdiv(R(1), rw + R(0.5));
+        if (sizeof(R) == 8) S.rw[threadIdx.x] = rw;
+    }
 }
 
 __device__ __forceinline__ int slot(int r) { return r & (RING - 1); }
@@ -120,14 +129,14 @@ __device__ __forceinline__ void load_rows(Core<R>& S, const R* in, int x0, int r
 }
 
 // mu_c = 2 beta C (C-1)(2C-1) - kappa lap C (reading R5) at ring offset s0
-// (column gx of the domain) with the y-neighbours at sN, sS.  The Laplacian
-// is the 5-point one, or in an axisymmetric domain the conservative
-// (1/r) d/dr (r dC/dr) + d2C/dz2 with faces at r = gx and gx + 1.
+// with the y-neighbours at sN, sS.  The Laplacian is the 5-point one, or in an
+// axisymmetric domain the conservative (1/r) d/dr (r dC/dr) + d2C/dz2 with
+// faces at r = rw and rw + 1.
 template <class R, bool AXI>
-__device__ __forceinline__ R chem_potential_of(const Consts<R>& K, R c, R ce, R cw, R cn, R cs, int gx, R inv_rc) {
+__device__ __forceinline__ R chem_potential_of(const Consts<R>& K, R c, R ce, R cw, R cn, R cs, R rw, R inv_rc) {
     R lap;
     if (AXI) {
-        const R rw = (R)gx, re = rw + R(1);
+        const R re = rw + R(1);
         lap = fma(re * (ce - c) - rw * (c - cw), inv_rc, cn + cs - R(2) * c);
     } else {
         lap = ce + cw + cn + cs - R(4) * c;
@@ -139,8 +148,8 @@ __device__ __forceinline__ R chem_potential_of(const Consts<R>& K, R c, R ce, R 
 template <class R, bool AXI>
 __device__ __forceinline__ R chem_potential(const Core<R>& S, int cc, int sc, int sN, int sS, int x0) {
     const P2<R>* RC = &S.P.rc[0][0];
-    return chem_potential_of<R, AXI>(S.K, RC[sc].y, RC[sc + 1].y, RC[sc - 1].y, RC[sN].y, RC[sS].y, x0 + cc - kHalo,
-                                     AXI ? S.inv_rc[cc] : R(0));
+    return chem_potential_of<R, AXI>(S.K, RC[sc].y, RC[sc + 1].y, RC[sc - 1].y, RC[sN].y, RC[sS].y,
+                                     AXI ? left_radius(S, cc, x0 + cc - kHalo) : R(0), AXI ? S.inv_rc[cc] : R(0));
 }
 
 // True if mu_c of rows [r0, r0 + nrows) of the strip involves no wall ghost
@@ -591,7 +600,7 @@ __device__ __forceinline__ void x_face(Core<R>& S, int x0, int r, int row_in_chu
     x.Lm = slot(r - 1) * RW + cL;
     x.Rp = x.Lp + 1;
     x.Rm = x.Lm + 1;
-    const R rf = AXI ? (R)(x0 + lane) : R(1);
+    const R rf = AXI ? left_radius(S, lane + kHalo, x0 + lane) : R(1);
     FaceFlux<R> F = GEN ? face_flux_gen<R, AXI>(S.K, S.P, x, true, true, inv_rf)
                         : face_flux<R, AXI>(S.K, S.P, x, true, true, inv_rf);
     if (AXI) {
@@ -701,15 +710,24 @@ __device__ __forceinline__ void cell_update(Core<R>& S, const Cell& in, int stag
     const SV<R> ws = stage == 0 ? wn : in.ws();
     SV<R> o;
     if constexpr (sizeof(R) == 8) {
-        // Eq. 58 as written
-        const R A = stage == 0 ? R(1) : (stage == 1 ? R(0.75) : R(1.0 / 3.0));
-        const R B = stage == 0 ? R(0) : (stage == 1 ? R(0.25) : R(2.0 / 3.0));
-        const R Cd = (stage == 0 ? R(1) : (stage == 1 ? R(0.25) : R(2.0 / 3.0))) * c2.z;
-        o.Hh = A * wn.Hh + B * ws.Hh + Cd * Rk[0];
-        o.p = A * wn.p + B * ws.p + Cd * Rk[1];
-        o.mx = A * wn.mx + B * ws.mx + Cd * Rk[2];
-        o.my = A * wn.my + B * ws.my + Cd * Rk[3];
-        o.Ch = A * wn.Ch + B * ws.Ch + Cd * Rk[4];
+        // Eq. 58 as written (stage 0 without its products by 1 and 0); explicit
+        // FMAs, so that both kernels round alike
+        if (stage == 0) {
+            o.Hh = fma(c2.z, Rk[0], wn.Hh);
+            o.p = fma(c2.z, Rk[1], wn.p);
+            o.mx = fma(c2.z, Rk[2], wn.mx);
+            o.my = fma(c2.z, Rk[3], wn.my);
+            o.Ch = fma(c2.z, Rk[4], wn.Ch);
+        } else {
+            const R A = stage == 1 ? R(0.75) : R(1.0 / 3.0);
+            const R B = stage == 1 ? R(0.25) : R(2.0 / 3.0);
+            const R Cd = B * c2.z;
+            o.Hh = fma(Cd, Rk[0], fma(A, wn.Hh, B * ws.Hh));
+            o.p = fma(Cd, Rk[1], fma(A, wn.p, B * ws.p));
+            o.mx = fma(Cd, Rk[2], fma(A, wn.mx, B * ws.mx));
+            o.my = fma(Cd, Rk[3], fma(A, wn.my, B * ws.my));
+            o.Ch = fma(Cd, Rk[4], fma(A, wn.Ch, B * ws.Ch));
+        }
         o.Hl = R(0);
         o.Cl = R(0);
     } else {
@@ -730,13 +748,13 @@ __device__ __forceinline__ void cell_update(Core<R>& S, const Cell& in, int stag
     }
     if (K.zsv) {   // reading R15: no motion of the solid part
         R Tn, Fln;
-        const R Cn = o.Ch + o.Cl;
+        const R Cn = pair_sum(o.Ch, o.Cl);
         invert_enthalpy(K, o.Hh, o.Hl, clamp01(Cn), Tn, Fln);
         const R keep = R(1) - solid_gate(K, Cn) * (R(1) - Fln);
         o.mx *= keep;
         o.my *= keep;
     }
-    if (!(isfinite(o.Hh) && isfinite(o.p) && isfinite(o.mx) && isfinite(o.my) && isfinite(o.Ch))) {
+    if (!(is_finite(o.Hh) && is_finite(o.p) && is_finite(o.mx) && is_finite(o.my) && is_finite(o.Ch))) {
         atomicOr(flag, 1);      // solver-wide
         atomicOr(K.flag, 1);    // this domain
     }

@@ -137,7 +137,7 @@ __device__ __forceinline__ SV<R> ring_cell(ShortSmem<R>& S, const R* in, int gx,
     }
     const SV<R> w = load_state(in, K.plane, (long long)sy * K.nx + sx + K.off);
     if (outer) {
-        R C = w.Ch + w.Cl;
+        R C = pair_sum(w.Ch, w.Cl);
         if (kx) C = ghost_C(K, sdx, kx, wall_wetting(K, in, sdx, sy), C);
         if (ky) C = ghost_C(K, sdy, ky, wall_wetting(K, in, sdy, gx), C);
         S.P.rc[slot(gy)][cc].y = C;
