@@ -123,19 +123,21 @@ __device__ __forceinline__ void invert_enthalpy(const Consts<R>& K, R Hh, R Hl, 
     const R Hs = cps * e.x;
     const R ds = pair_sum(Hh - Hs, Hl);
     const R dl = pair_sum(Hh - HL, Hl);
-    if (negative(ds)) {
-        Fl = R(0);
-        T = wdiv(pair_sum(Hh, Hl), cps);
-    } else if (positive(dl)) {
-        Fl = R(1);
-        T = e.y + wdiv(dl, cpl);
-    } else if (positive(HL - Hs)) {
-        Fl = wdiv(ds, HL - Hs);
-        T = fma(Fl, e.w, e.x);
-    } else {
-        Fl = R(1);
-        T = e.y;
-    }
+    // one division whichever branch a cell takes: a warp with cells on several
+    // branches passes it once, and the code has no divergent paths.  us per step: 64
+    // domains 1021 -> 1006, 512^2 54.1 -> 53.2, 128^2 14.0 -> 13.9; FP64 16 domains
+    // 4711 -> 4702.  (Choosing num and den by selects keeps more registers live: the
+    // two-per-SM short kernel spilled 28 bytes and lost 0.5 %.)
+    const bool solid = negative(ds), liquid = positive(dl);
+    R num = ds, den = HL - Hs;
+    if (!positive(den)) { num = R(1); den = R(1); }
+    if (liquid) { num = dl; den = cpl; }
+    if (solid) { num = pair_sum(Hh, Hl); den = cps; }
+    const R q = wdiv(num, den);
+    Fl = q;
+    T = fma(q, e.w, e.x);
+    if (liquid) { Fl = R(1); T = e.y + q; }
+    if (solid) { Fl = R(0); T = q; }
 }
 
 // Eq. 7 as m.x + X (m.y + Y m.z).  Reading R1: gamma = C~ [F_s g_s + F_l g_l]
