@@ -55,6 +55,12 @@ __device__ __forceinline__ void store_state(float* b, long long P, long long c, 
     b[5 * P + c] = s.Ch; b[6 * P + c] = s.Cl;
 }
 
+// A product and a sum that the compiler may not fuse with what follows or comes
+// before: the stage kernels inline the same expressions, and have to round alike.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+
 // Knuth's TwoSum: s + e == a + b exactly.
 template <class R>
 __device__ __forceinline__ void two_sum(R a, R b, R& s, R& e) {
@@ -136,7 +142,7 @@ __device__ __forceinline__ void invert_enthalpy(const Consts<R>& K, R Hh, R Hl, 
     const R q = wdiv(num, den);
     Fl = q;
     T = fma(q, e.w, e.x);
-    if (liquid) { Fl = R(1); T = e.y + q; }
+    if (liquid) { Fl = R(1); T = add_rn(e.y, q); }
     if (solid) { Fl = R(0); T = q; }
 }
 

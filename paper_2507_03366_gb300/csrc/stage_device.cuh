@@ -137,12 +137,13 @@ __device__ __forceinline__ R chem_potential_of(const Consts<R>& K, R c, R ce, R 
     R lap;
     if (AXI) {
         const R re = rw + R(1);
-        lap = fma(re * (ce - c) - rw * (c - cw), inv_rc, cn + cs - R(2) * c);
+        lap = fma(fma(re, ce - c, -(rw * (c - cw))), inv_rc, fma(R(-2), c, cn + cs));
     } else {
-        lap = ce + cw + cn + cs - R(4) * c;
+        lap = fma(R(-4), c, ce + cw + cn + cs);
     }
     const Q4<R> cc = ld4(K.cellc2);   // 2 beta, kappa
-    return cc.x * c * (c - R(1)) * (R(2) * c - R(1)) - cc.y * lap;
+    // (explicit FMAs: every place that inlines this has to round alike)
+    return fma(-cc.y, lap, cc.x * c * (c - R(1)) * fma(R(2), c, R(-1)));
 }
 
 template <class R, bool AXI>
@@ -737,8 +738,8 @@ __device__ __forceinline__ void cell_update(Core<R>& S, const Cell& in, int stag
         // every pair canonical.
         R dH, dC;
         if (stage == 0) {
-            dH = c2.z * Rk[0];
-            dC = c2.z * Rk[4];
+            dH = mul_rn(c2.z, Rk[0]);
+            dC = mul_rn(c2.z, Rk[4]);
             o.p = fma(c2.z, Rk[1], wn.p);
             o.mx = fma(c2.z, Rk[2], wn.mx);
             o.my = fma(c2.z, Rk[3], wn.my);
