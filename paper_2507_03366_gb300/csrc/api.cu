@@ -420,6 +420,32 @@ int short_rows(const eulbfs_solver* s, bool fp64) {
     return best;
 }
 
+// The runs of rows that the tiled kernel cuts a domain into, at a target height.
+int tiled_runs(int ny, int rows) {
+    const int chunks = (ny + kChunk - 1) / kChunk, per = std::max(1, rows / kChunk);
+    return std::min(chunks, std::max(1, (chunks + per / 2) / per));
+}
+
+// Split domains exchange halos between the stages: one launch per stage, as with
+// eulbfs_set_whole_step(0).
+bool launch_per_stage(const eulbfs_solver* s) {
+    if (!s->whole_step) return true;
+    const int nd = (int)s->doms.size();
+    for (const int2& l : s->links)
+        if (l.x < nd && l.y < nd && s->doms[l.x].active() && s->doms[l.y].active()) return true;
+    return false;
+}
+
+// A launch per stage ends with its last item, so where items of up to this many
+// rows make one wave of the tiled kernel's resident CTAs, the shortest such are
+// taken.  us per step of droplets in slabs, with the rule for whole-step launches and
+// in one wave: 400^2 in two 71.6 (8 rows) -> 69.4 (16), 512^2 in two 80.5 (8) -> 72.8
+// (16), 600^2 in two 99.9 (8) -> 96.9 (24), 640^2 in four 126.7 (16) -> 99.7 (24),
+// 768^2 in four 131.0 (16) -> 127.3 (32); FP64 512^2 1125 (16) -> 1087 (32).  Beyond,
+// several waves are better: 900^2 in four 176.6 (24; one wave of 48: 180.3),
+// 1024^2 in three 217 (24; 64: 241).
+constexpr int kOneWaveRows = 32;
+
 ItemPlan plan_items(const eulbfs_solver* s) {
     const bool fp64 = s->precision == EULBFS_FP64;
     long long strip_rows = 0;   // rows of all strips
@@ -427,7 +453,15 @@ ItemPlan plan_items(const eulbfs_solver* s) {
         if (d.active()) strip_rows += (long long)((d.grid.nx + kStripX - 1) / kStripX) * d.grid.ny;
     // input tiles, and so the probe of their waits, are the tiled kernel's
     if (!s->tile_probe && strip_rows * 10 <= 41LL * s->sms * kShortRows) return ItemPlan{true, short_rows(s, fp64)};
-    const long long wave = (long long)stage_blocks_per_sm(s->precision) * s->sms * kChunk;
+    const long long resident = (long long)stage_blocks_per_sm(s->precision) * s->sms;
+    if (launch_per_stage(s))
+        for (int rows = kChunk; rows <= std::min(kOneWaveRows, s->seg); rows += kChunk) {
+            long long n = 0;
+            for (const Dom& d : s->doms)
+                if (d.active()) n += (long long)((d.grid.nx + kStripX - 1) / kStripX) * tiled_runs(d.grid.ny, rows);
+            if (n <= resident) return ItemPlan{false, rows};
+        }
+    const long long wave = resident * kChunk;
     const long long chunks = (strip_rows * 10 + 26 * wave - 1) / (26 * wave);
     return ItemPlan{false, (int)std::min<long long>(s->seg / kChunk, std::max(1LL, chunks)) * kChunk};
 }
@@ -474,7 +508,7 @@ int rebuild(eulbfs_solver* s) {
         const int chunks = (d.grid.ny + unit - 1) / unit, per = std::max(1, plan.rows / unit);
         d.desc.strips = (d.grid.nx + kStripX - 1) / kStripX;
         d.desc.segs = plan.short_items ? (chunks + per - 1) / per
-                                       : std::min(chunks, std::max(1, (chunks + per / 2) / per));
+                                       : tiled_runs(d.grid.ny, plan.rows);
         if (!d.active()) continue;
         for (int sy = 0; sy < d.desc.segs; ++sy) {
             const int y0 = (int)((long long)sy * chunks / d.desc.segs) * unit;
@@ -486,17 +520,13 @@ int rebuild(eulbfs_solver* s) {
     // (short items are of one height within a row, and stay in row order: the
     // next stage's first items then wait for items claimed long before)
     if (!plan.short_items) std::stable_sort(items.begin(), items.end(), taller);
-    // launches per stage (split domains exchange halos between stages, or
-    // eulbfs_set_whole_step(0)): the end of the list in shorter items --
+    // launches per stage: the end of the list in shorter items --
     // kTailLevels times, the last wave (one item per resident CTA) is cut in
     // half, so each launch ends on items 2^-kTailLevels as tall and the first
     // CTAs to run out of work wait less for the last.  A whole-step launch
     // has no stage ends to shorten (the next stage's items fill them), and
     // its one end gains less than the extra prologues cost.
-    bool linked = false;
-    for (const int2& l : s->links)
-        linked |= l.x < nd && l.y < nd && s->doms[l.x].active() && s->doms[l.y].active();
-    const int tail_levels = plan.short_items || (s->whole_step && !linked) ? 0 : kTailLevels;
+    const int tail_levels = plan.short_items || !launch_per_stage(s) ? 0 : kTailLevels;
     const int resident = stage_blocks_per_sm(s->precision) * s->sms;
     for (int level = 0; level < tail_levels && (long long)items.size() > 2LL * resident; ++level) {
         std::vector<int4> tail;
