@@ -123,6 +123,31 @@ struct SharedCell {
     __device__ __forceinline__ SV<R> ws() const { return get_cell(S.ws, row, lane); }
 };
 
+// The halo of an item, narrowing away from its rows: what is read of the rows at
+// distance 1 are ring columns 1 .. RW-2 (mu_c of the item's own end columns), at
+// distance 2 columns 2 .. RW-3 and at distance 3 columns 3 .. RW-4 (C alone).  So
+// an item of 8 rows has 37 x 8 + 198 = 494 cells, one for each of the 512 threads;
+// the rectangle's 518 took one warp through a second round of loads.
+// us per step: 400x200 22.8 -> 21.6, 333x251 22.4 -> 21.7, 256^2 20.1 (both).  Lower
+// items and FP64 (bound by its arithmetic) keep the rectangle, whose indices are
+// quicker: 1024x4 in one-row items 12.3, narrowing 12.6; FP64 256x4 44.7 (44.9).
+template <class R, int PER_SM>
+constexpr bool kNarrow = sizeof(R) == 4 && PER_SM == 2;
+constexpr int kHalo1 = 2 * (RW - 2), kHalo2 = kHalo1 + 2 * (RW - 4), kHaloCells = kHalo2 + 2 * (RW - 6);
+
+// Halo cell j of an item of `rows` rows: its row relative to the item's first, its
+// ring column, and whether it lies at distance 3.
+__device__ __forceinline__ bool halo_cell(int j, int rows, int& rr, int& cc) {
+    int d = 1;
+    if (j >= kHalo1) { d = 2; j -= kHalo1; }
+    if (d == 2 && j >= kHalo2 - kHalo1) { d = 3; j -= kHalo2 - kHalo1; }
+    const int w = RW - 2 * d;
+    const bool above = j >= w;
+    cc = d + (above ? j - w : j);
+    rr = above ? rows - 1 + d : -d;
+    return d == 3;
+}
+
 // Load and derive cell (gx, gy) into ring column cc; a halo cell outside the
 // domain is mapped through the boundary rules (as load_rows).  Of the outer
 // rows (the third halo row on both sides) only C is ever read, by mu_c.
@@ -155,7 +180,7 @@ __device__ __forceinline__ SV<R> ring_cell(ShortSmem<R>& S, const R* in, int gx,
 
 // One work item: rows [y0, y1) (at most kShortRows) of the strip at x0.
 // `claim`: the control warp's claimed next position, looked up in here.
-template <class R, bool AXI, bool GEN, int NTS>
+template <class R, bool AXI, bool GEN, int NTS, bool NARROW>
 __device__ __forceinline__ void short_item(ShortSmem<R>& S, const StageLaunch& a, const int stage, int x0, int y0,
                                            int y1, int claim) {
     constexpr int NWS = NTS / 32;
@@ -177,13 +202,16 @@ __device__ __forceinline__ void short_item(ShortSmem<R>& S, const StageLaunch& a
     }
     // ... and the rows with their halo
     const bool inside = x0 >= kHalo && x0 + kStripX + kHalo <= K.nx && y0 - kHalo >= -K.hlo && y1 + kHalo <= K.ny + K.hhi;
-    const int total = (rows + 2 * kHalo) * RW;
-    for (int idx = tid; idx < total; idx += NTS) {
-        const int rr = idx / RW, cc = idx - rr * RW;
-        const SV<R> w = ring_cell(S, in, x0 + cc - kHalo, y0 + rr - kHalo, cc, inside,
-                                  rr == 0 || rr == rows + 2 * kHalo - 1);
-        const int ir = rr - kHalo, ic = cc - kHalo;
-        if (ir >= 0 && ir < rows && ic >= 0 && ic < kStripX) put_cell(S.ws, ir, ic, w);
+    constexpr int low = NARROW ? 0 : -kHalo;   // the first row that comes whole
+    const int own = (rows - 2 * low) * RW;
+    for (int idx = tid; idx < own + (NARROW ? kHaloCells : 0); idx += NTS) {
+        int rr = idx / RW, cc = idx - rr * RW;
+        rr += low;
+        bool outer = !NARROW && (rr == -kHalo || rr == rows + kHalo - 1);
+        if (NARROW && idx >= own) outer = halo_cell(idx - own, rows, rr, cc);
+        const SV<R> w = ring_cell(S, in, x0 + cc - kHalo, y0 + rr, cc, inside, outer);
+        const int ic = cc - kHalo;
+        if (rr >= 0 && rr < rows && ic >= 0 && ic < kStripX) put_cell(S.ws, rr, ic, w);
     }
     if (upd) {
         S.frac[ur][ul] = fr;
@@ -192,6 +220,8 @@ __device__ __forceinline__ void short_item(ShortSmem<R>& S, const StageLaunch& a
     const R ir_c = AXI ? wdiv(R(1), (R)(x0 + lane) + R(0.5)) : R(1);
     const R ir_f = (AXI && x0 + lane > 0) ? wdiv(R(1), (R)(x0 + lane)) : R(0);
     __syncthreads();
+    // (of a halo that narrows, the end columns on either side take values of cells
+    // that were not loaded; nothing reads those)
     muc_rows<R, AXI, NTS>(S, x0, y0 - 2, rows + 4);
     __syncthreads();
     if (warp == NWS - 1) look_up(S, a, __shfl_sync(0xffffffffu, claim, 0), lane);
@@ -270,11 +300,11 @@ __global__ void __launch_bounds__(kThreads<R, PER_SM>, PER_SM) short_kernel(Stag
         const int x0 = item.y * kStripX;
         const int stage = st % 3;
         if (S.K.gen) {
-            if (S.K.axi) short_item<R, true, true, NTS>(S, a, stage, x0, item.z, item.w, claim);
-            else short_item<R, false, true, NTS>(S, a, stage, x0, item.z, item.w, claim);
+            if (S.K.axi) short_item<R, true, true, NTS, kNarrow<R, PER_SM>>(S, a, stage, x0, item.z, item.w, claim);
+            else short_item<R, false, true, NTS, kNarrow<R, PER_SM>>(S, a, stage, x0, item.z, item.w, claim);
         } else {
-            if (S.K.axi) short_item<R, true, false, NTS>(S, a, stage, x0, item.z, item.w, claim);
-            else short_item<R, false, false, NTS>(S, a, stage, x0, item.z, item.w, claim);
+            if (S.K.axi) short_item<R, true, false, NTS, kNarrow<R, PER_SM>>(S, a, stage, x0, item.z, item.w, claim);
+            else short_item<R, false, false, NTS, kNarrow<R, PER_SM>>(S, a, stage, x0, item.z, item.w, claim);
         }
         const int rows = item.w - item.z;
         if (a.stages > 1 && warp < rows && !a.dep_probe) {
