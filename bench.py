@@ -45,10 +45,10 @@ BYTES_STAGE_BY_STAGE = {1: 244, 0: 352}
 # (FP64: 2 steps), planar and axisymmetric): per cell and stage, FP32 (FP64)
 # operations with an FMA counted as 2 and warp instructions issued; per
 # cell and step, DRAM bytes.  They belong to one version of the kernel's sources: the
-# SHA-256 of stage.cu + device_common.cuh + eulbfs_internal.h.  When the
+# SHA-256 of KERNEL_SOURCES, in that order.  When the
 # sources change, the counters are reported as stale (null) until they are
 # captured again.
-KERNEL_SOURCES = ("stage.cu", "device_common.cuh", "eulbfs_internal.h")
+KERNEL_SOURCES = ("stage.cu", "stage_device.cuh", "device_common.cuh", "eulbfs_internal.h")
 COUNTERS = {
     "sources_sha256": "cbface8b97d14d2489ffbb3e171fe71d595a2fff85d003d3b12838e4224168c8",
     "fp32_flops_per_cell_stage": {"rz": 942.3, "xy": 905.0},

@@ -386,15 +386,15 @@ struct ItemPlan {
 // upper limit).  us per step on one GB300, FP32C unless marked; 64: the height
 // that every batch once had:
 //   - the short-item kernel, up to 4.1 items of kShortRows rows per SM: 128^2
-//     121 (64) -> 14.3, 400x200 193 -> 23, 333x251 131 -> 23, 1024x4 27 -> 12.9;
-//     FP64 256x4 135 -> 50, 128^2 1281 -> 115, 256^2 1326 -> 292 (the tiled
+//     121 (64) -> 13.9, 400x200 193 -> 21.6, 333x251 131 -> 21.6, 1024x4 27 -> 12.3;
+//     FP64 256x4 135 -> 44.7, 128^2 1281 -> 108, 256^2 1326 -> 277 (the tiled
 //     kernel in 8-row items: 31, 37, 34, 26; FP64 135, 192, 340).  At the limit
 //     the two meet: 384^2 39 (tiled 43), 448^2 53 (50); FP64 384^2 590 (611);
 //   - else the tiled kernel with the tallest items that still make 2.6 waves of
-//     its resident CTAs, up to kDefaultRows: 512^2 148 (64) -> 64 (8 rows), 640^2
-//     165 -> 80 (16), 768^2 171 -> 106 (16), 1024^2 223 -> 176 (24; 32: 168,
-//     16: 192), 16 droplet domains 265 -> 260 (40), 64 domains 941 -> 914 (128;
-//     160: 927).
+//     its resident CTAs, up to kDefaultRows: 512^2 54 (8 rows; 16: 58, 64: 126),
+//     640^2 70 (16; 8: 79, 64: 147), 1024^2 155 (24; 16: 164, 32: 151, 64: 208),
+//     16 droplet domains 214 (32; 24: 225, 40: 219, 64: 227), 64 domains 914 (128;
+//     160: 927, 64: 941).
 // The height of short items: the one with the least work for the busiest SM.  An
 // item of h rows costs as b + h (a stage of one FP64 item keeps its SM's pipe
 // busy for about 8 + 9 h thousand clocks, whoever shares the SM; fitted for
