@@ -50,11 +50,11 @@ BYTES_STAGE_BY_STAGE = {1: 244, 0: 352}
 # captured again.
 KERNEL_SOURCES = ("stage.cu", "stage_device.cuh", "device_common.cuh", "eulbfs_internal.h")
 COUNTERS = {
-    "sources_sha256": "cbface8b97d14d2489ffbb3e171fe71d595a2fff85d003d3b12838e4224168c8",
-    "fp32_flops_per_cell_stage": {"rz": 942.3, "xy": 905.0},
-    "warp_inst_per_cell_stage": {"rz": 44.84, "xy": 43.53},
-    "dram_bytes_per_cell_step": {"rz": 350.6, "xy": 345.1},
-    "fp64_flops_per_cell_stage": {"rz": 1011.7, "xy": 940.4},
+    "sources_sha256": "3e8740e0d72976c341ede07b61cfbc0a4810b5cfee0f35344e95461376d41309",
+    "fp32_flops_per_cell_stage": {"rz": 815.2, "xy": 777.8},
+    "warp_inst_per_cell_stage": {"rz": 41.37, "xy": 40.22},
+    "dram_bytes_per_cell_step": {"rz": 360.0, "xy": 356.7},
+    "fp64_flops_per_cell_stage": {"rz": 853.8, "xy": 815.1},
 }
 # Streaming steps (dt_h, dt_f, dt_g) of the general-face-path leg.
 GEN_STEPS = (0.3, 0.4, 0.3)
