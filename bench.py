@@ -50,10 +50,10 @@ BYTES_STAGE_BY_STAGE = {1: 244, 0: 352}
 # captured again.
 KERNEL_SOURCES = ("stage.cu", "stage_device.cuh", "device_common.cuh", "eulbfs_internal.h")
 COUNTERS = {
-    "sources_sha256": "3e8740e0d72976c341ede07b61cfbc0a4810b5cfee0f35344e95461376d41309",
-    "fp32_flops_per_cell_stage": {"rz": 815.2, "xy": 777.8},
-    "warp_inst_per_cell_stage": {"rz": 41.37, "xy": 40.22},
-    "dram_bytes_per_cell_step": {"rz": 360.0, "xy": 356.7},
+    "sources_sha256": "85c0dc1f2c3fe86265056518fb83efd139388e20014246632c615285c7176b71",
+    "fp32_flops_per_cell_stage": {"rz": 818.1, "xy": 780.7},
+    "warp_inst_per_cell_stage": {"rz": 41.54, "xy": 40.41},
+    "dram_bytes_per_cell_step": {"rz": 357.0, "xy": 352.2},
     "fp64_flops_per_cell_stage": {"rz": 853.8, "xy": 815.1},
 }
 # Streaming steps (dt_h, dt_f, dt_g) of the general-face-path leg.

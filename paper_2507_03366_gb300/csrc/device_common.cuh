@@ -58,7 +58,6 @@ __device__ __forceinline__ void store_state(float* b, long long P, long long c, 
 // A product and a sum that the compiler may not fuse with what follows or comes
 // before: the stage kernels inline the same expressions, and have to round alike.
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 
 // Knuth's TwoSum: s + e == a + b exactly.
@@ -102,6 +101,19 @@ __device__ __forceinline__ double pair_sum(double hi, double) { return hi; }
 __device__ __forceinline__ double wdiv(double a, double b) { return a / b; }
 __device__ __forceinline__ float wdiv(float a, float b) { return __fdividef(a, b); }
 
+// num / den, and base + num / den with one rounding after the reciprocal's (FP64: the
+// quotient's and the sum's).
+__device__ __forceinline__ float quotient(float num, float den, float base, float& sum) {
+    const float r = wdiv(1.0f, den);
+    sum = fma(num, r, base);
+    return mul_rn(num, r);
+}
+__device__ __forceinline__ double quotient(double num, double den, double base, double& sum) {
+    const double q = wdiv(num, den);
+    sum = add_rn(base, q);
+    return q;
+}
+
 // Eq. 5-6 with the readings of the oracle: uniform latent heat, Eq. 7 mixture
 // heat capacity gated by clamp(C).  H = Hh + Hl (Hl = 0 in FP64); the
 // differences H - H_s and H - H_l are formed from the pair without rounding H.
@@ -139,10 +151,11 @@ __device__ __forceinline__ void invert_enthalpy(const Consts<R>& K, R Hh, R Hl, 
     if (!positive(den)) { num = R(1); den = R(1); }
     if (liquid) { num = dl; den = cpl; }
     if (solid) { num = pair_sum(Hh, Hl); den = cps; }
-    const R q = wdiv(num, den);
+    R above;   // T_l + num / den; in FP32 without rounding the quotient
+    const R q = quotient(num, den, e.y, above);
     Fl = q;
     T = fma(q, e.w, e.x);
-    if (liquid) { Fl = R(1); T = add_rn(e.y, q); }
+    if (liquid) { Fl = R(1); T = above; }
     if (solid) { Fl = R(0); T = q; }
 }
 
