@@ -12,9 +12,6 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>   // header-only: ranges cost a pointer test unless a profiler is attached
 
-#include <sys/mman.h>
-#include <unistd.h>
-
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -24,6 +21,7 @@
 
 #include "eulbfs.h"
 #include "eulbfs_internal.h"
+#include "host_pages.h"
 
 using namespace eulbfs;
 
@@ -48,25 +46,6 @@ int cuda_fail(cudaError_t e, const char* what) {
 
 constexpr double kDtStream = 0.5;   // c dt_s = dx / 2 (Sec. 2.5 step (1))
 constexpr int kMinSlabRows = 8;     // interior rows of each slab of a split domain
-
-#ifndef MADV_POPULATE_WRITE
-#define MADV_POPULATE_WRITE 23
-#endif
-
-// Map the pages of a host output buffer before the GPU writes to it.  A fresh
-// allocation (a bytes object, numpy.empty) has none yet, and on a host whose
-// pageable memory the GPU reaches directly the copy faults them in one by one:
-// checkpoints of 64 domains (231 MB) took 121 ms, and take 12.5.
-void map_output(void* p, size_t bytes) {
-    constexpr size_t kLeast = 1 << 16;   // smaller buffers come from pages in use
-    if (!p || bytes < kLeast) return;
-    const size_t page = (size_t)sysconf(_SC_PAGESIZE);
-    const uintptr_t a = reinterpret_cast<uintptr_t>(p) / page * page;
-    if (madvise(reinterpret_cast<void*>(a), reinterpret_cast<uintptr_t>(p) + bytes - a, MADV_POPULATE_WRITE) == 0) return;
-    volatile char* c = static_cast<volatile char*>(p);   // an older kernel: touch every page
-    for (size_t k = 0; k < bytes; k += page) c[k] = 0;
-    c[bytes - 1] = 0;
-}
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
