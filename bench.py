@@ -251,7 +251,7 @@ def workload_config(cases, world: int, args) -> dict:
                         f"{{128,192,256,384,512}}, {cells} cells per GPU",
             "global_batch": len(cases) * world, "seq_len": cells, "parallelism": f"independent domains x{world}",
             "precision": "FP32C",
-            "work_item": (f"31-column strips, rows cut into runs of about {args.tile}"
+            "work_item": (f"31-column strips, rows cut into runs of about {getattr(args, 'rows', args.tile)}"
                           + (" (autotuned)" if getattr(args, "autotuned", False) else ""))
             if args.tile else "31-column strip segments, height autotuned", "graph_steps": args.graph,
             "launch": ("one per Runge-Kutta stage" if args.stage_launches else
@@ -387,11 +387,13 @@ def main():
     tuning = None
     if args.tile == 0:
         # the autotuner times each candidate height on the live batch (its
-        # steps are part of the warm-up); every solver below uses the winner
+        # steps are part of the warm-up) and keeps the best; the solvers of the
+        # other legs use the fastest candidate
         args.tile, _ = sol.autotune(5)
-        args.autotuned = True
+        args.autotuned, args.rows = True, sol.work_list()["rows"]
         tuning = {str(k): v for k, v in sorted(sol.autotune_report().items())}
-    sol.set_tile(args.tile)
+    else:
+        sol.set_tile(args.tile)
     sol.set_whole_step(not args.stage_launches)
     if args.graph:
         sol.use_graphs(args.graph)

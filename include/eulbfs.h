@@ -313,14 +313,22 @@ int eulbfs_set_whole_step(eulbfs_solver* s, int on);
 int eulbfs_use_graphs(eulbfs_solver* s, int steps_per_graph);
 
 /* Work-item shape of the stage kernels: each item is a 31-column strip of a
- * domain and a run of its rows.  `rows` (a multiple of 8 in [8, 1024];
- * 0 = 128, the default) is the largest target height: a domain of ny rows is
- * cut into round(ny / rows) runs (at least one) of nearly equal height, in
- * whole 8-row chunks, or into shorter ones (down to one row) where the batch
- * has too few cells to fill the GPU with items of that height.  The
- * persistent CTAs claim items from a counter, tallest first.  Results do not
- * depend on it. */
+ * domain and a run of its rows.  `rows` (a multiple of 8 in [8, 1024]) is the
+ * target height: a domain of ny rows is cut into round(ny / rows) runs (at
+ * least one) of nearly equal height, in whole 8-row chunks, whatever the size
+ * of the batch.  0 (the default): the height follows the batch, from 128 rows
+ * where it fills the GPU with items of that height down to one row where it
+ * has few cells.  The persistent CTAs claim items from a counter, tallest first
+ * (items of at most 8 rows in row order).  Results do not depend on it. */
 int eulbfs_set_tile(eulbfs_solver* s, int rows);
+
+/* The work list of the next step, for tests and tuning: *short_items receives 1
+ * if the batch runs in the kernel for short items (at most 8 rows), 0 for the
+ * one for taller ones; *rows the target height; *items how many there are;
+ * *ctas_per_sm the CTAs that share an SM.  Builds the list if domains or
+ * settings have changed since the last step (and then synchronises the solver's
+ * stream).  Any pointer may be NULL.  Errors: EINVAL, ECUDA. */
+int eulbfs_work_list(eulbfs_solver* s, int* short_items, int* rows, int* items, int* ctas_per_sm);
 
 /* Diagnostics of a caller-held domain state that allocates no device memory.
  * The paper has no counterpart to this call; it exists for callers that
@@ -356,12 +364,16 @@ int eulbfs_diagnostics_noalloc(int precision, const void* state, int nx, int ny,
 
 /* Pick the work-item height of the current batch by timing each candidate
  * (32, 48, 64, 96, 128, 160, 192, 256 rows) over steps_per_candidate steps on
- * the solver's stream, in two rounds, and keeping the candidate with the
- * fastest of its two timings (*best_ms_per_step).  The timed steps are real
- * steps of every active domain (results do not depend on the height), so the
- * simulation advances by 2 * 8 * (steps_per_candidate + 1) steps.  Synchronises the
- * stream.  EULBFS_EINVAL for a null solver or steps_per_candidate < 1; a
- * failing step returns its error and leaves the height unchanged. */
+ * the solver's stream, in two rounds.  The heights by the batch's size
+ * (eulbfs_set_tile(s, 0)) are timed in the second round, twice, in place of the
+ * two candidates that were slowest in the first.  *best_rows and
+ * *best_ms_per_step receive the candidate with the fastest of its timings; the
+ * solver takes that height if it is faster than the heights by the batch's size,
+ * and those otherwise.  The timed steps are real steps of every active domain
+ * (results do not depend on the height), so the simulation advances by
+ * 2 * 8 * (steps_per_candidate + 1) steps.  Synchronises the stream.
+ * EULBFS_EINVAL for a null solver or steps_per_candidate < 1; a failing step
+ * returns its error and leaves the height unchanged. */
 int eulbfs_autotune(eulbfs_solver* s, int steps_per_candidate, int* best_rows, float* best_ms_per_step);
 
 /* Test hook for the bounded device waits (no counterpart in the paper).
@@ -379,8 +391,8 @@ int eulbfs_autotune(eulbfs_solver* s, int steps_per_candidate, int* best_rows, f
 int eulbfs_set_tile_wait_probe(eulbfs_solver* s, int on);
 
 /* The candidates the last eulbfs_autotune of this solver timed: up to `cap`
- * heights (rows) and their best milliseconds per step; *n receives how many
- * it timed (0 before any autotune).  Errors: EINVAL (null solver or n,
+ * heights (rows) and their best milliseconds per step (of the candidates alone);
+ * *n receives how many it timed (0 before any autotune).  Errors: EINVAL (null solver or n,
  * cap < 0, null arrays with cap > 0). */
 int eulbfs_autotune_report(const eulbfs_solver* s, int* rows, float* ms_per_step, int cap, int* n);
 

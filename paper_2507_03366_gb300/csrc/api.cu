@@ -170,7 +170,7 @@ int eulbfs::set_error(int code, const char* msg) { return fail(code, msg); }
 
 constexpr int kMaxTune = 8;   // autotune candidates kept for eulbfs_autotune_report
 constexpr int kTailLevels = 2;   // halvings of the work list's last wave (launches per stage)
-constexpr int kDefaultRows = 128;   // tallest work item unless eulbfs_set_tile says otherwise
+constexpr int kDefaultRows = 128;   // tallest work item of a batch whose heights follow its size
 constexpr int kMaxLaunchSteps = 16;   // time steps in one whole-step launch at most
 
 struct eulbfs_solver {
@@ -186,8 +186,9 @@ struct eulbfs_solver {
     int items_cap = 0;
     int nitems = 0;
     bool short_items = false;      // the work list is for the short-item kernel
+    int item_rows = 0;             // its target height
     bool dirty = true;
-    int seg = kDefaultRows;        // tallest work item (rows)
+    int seg = 0;                   // target rows of a work item (eulbfs_set_tile); 0: by the batch's size
     int sms = 1;
     int grid = 1;
     int* d_flag = nullptr;
@@ -361,8 +362,8 @@ struct ItemPlan {
 
 // How the active domains' rows are cut into work items.  A stage cannot end
 // before its tallest item does, and an item of many rows is a long serial
-// sweep, so a batch that does not fill the chip is cut finer (s->seg stays the
-// upper limit).  us per step on one GB300, FP32C unless marked; 64: the height
+// sweep, so a batch that does not fill the chip is cut finer, unless
+// eulbfs_set_tile names a height (s->seg).  us per step on one GB300, FP32C unless marked; 64: the height
 // that every batch once had:
 //   - the short-item kernel, up to 4.1 items of kShortRows rows per SM: 128^2
 //     121 (64) -> 13.9, 400x200 193 -> 21.6, 333x251 131 -> 21.6, 1024x4 27 -> 12.3;
@@ -426,6 +427,7 @@ bool launch_per_stage(const eulbfs_solver* s) {
 constexpr int kOneWaveRows = 32;
 
 ItemPlan plan_items(const eulbfs_solver* s) {
+    if (s->seg) return ItemPlan{false, s->seg};
     const bool fp64 = s->precision == EULBFS_FP64;
     long long strip_rows = 0;   // rows of all strips
     for (const Dom& d : s->doms)
@@ -434,7 +436,7 @@ ItemPlan plan_items(const eulbfs_solver* s) {
     if (!s->tile_probe && strip_rows * 10 <= 41LL * s->sms * kShortRows) return ItemPlan{true, short_rows(s, fp64)};
     const long long resident = (long long)stage_blocks_per_sm(s->precision) * s->sms;
     if (launch_per_stage(s))
-        for (int rows = kChunk; rows <= std::min(kOneWaveRows, s->seg); rows += kChunk) {
+        for (int rows = kChunk; rows <= kOneWaveRows; rows += kChunk) {
             long long n = 0;
             for (const Dom& d : s->doms)
                 if (d.active()) n += (long long)((d.grid.nx + kStripX - 1) / kStripX) * tiled_runs(d.grid.ny, rows);
@@ -442,7 +444,7 @@ ItemPlan plan_items(const eulbfs_solver* s) {
         }
     const long long wave = resident * kChunk;
     const long long chunks = (strip_rows * 10 + 26 * wave - 1) / (26 * wave);
-    return ItemPlan{false, (int)std::min<long long>(s->seg / kChunk, std::max(1LL, chunks)) * kChunk};
+    return ItemPlan{false, (int)std::min<long long>(kDefaultRows / kChunk, std::max(1LL, chunks)) * kChunk};
 }
 
 int rebuild(eulbfs_solver* s) {
@@ -476,6 +478,7 @@ int rebuild(eulbfs_solver* s) {
     }
     const ItemPlan plan = plan_items(s);
     s->short_items = plan.short_items;
+    s->item_rows = plan.rows;
     // work items: each domain's rows (in whole kChunk-row chunks for the tiled
     // kernel) split into runs of nearly equal length; the list runs the
     // tallest items first, so that the persistent CTAs, which claim items in
@@ -878,8 +881,7 @@ int eulbfs_domain_progress(const eulbfs_solver* s, int slot, long long* done, lo
 
 int eulbfs_set_tile(eulbfs_solver* s, int rows) {
     if (!s) return fail(EULBFS_EINVAL, "null solver");
-    if (rows == 0) rows = kDefaultRows;
-    if (rows < kChunk || rows > 1024 || rows % kChunk) return fail(EULBFS_EINVAL, "segment height must be a multiple of 8 in [8, 1024]");
+    if (rows != 0 && (rows < kChunk || rows > 1024 || rows % kChunk)) return fail(EULBFS_EINVAL, "segment height must be a multiple of 8 in [8, 1024]");
     if (rows != s->seg) {
         s->seg = rows;
         s->dirty = true;
@@ -887,39 +889,64 @@ int eulbfs_set_tile(eulbfs_solver* s, int rows) {
     return EULBFS_OK;
 }
 
+int eulbfs_work_list(eulbfs_solver* s, int* short_items, int* rows, int* items, int* ctas_per_sm) {
+    if (!s) return fail(EULBFS_EINVAL, "null solver");
+    if (s->dirty) {
+        int rc = rebuild(s);
+        if (rc) return rc;
+    }
+    if (short_items) *short_items = s->short_items;
+    if (rows) *rows = s->item_rows;
+    if (items) *items = s->nitems;
+    if (ctas_per_sm)
+        *ctas_per_sm = !s->short_items ? stage_blocks_per_sm(s->precision)
+                       : s->grid <= s->sms ? 1 : short_blocks_per_sm(s->precision);
+    return EULBFS_OK;
+}
+
 int eulbfs_autotune(eulbfs_solver* s, int steps_per_candidate, int* best_rows, float* best_ms_per_step) {
     if (!s) return fail(EULBFS_EINVAL, "null solver");
     if (steps_per_candidate < 1) return fail(EULBFS_EINVAL, "steps_per_candidate must be >= 1");
     static const int kCandidates[] = {32, 48, 64, 96, 128, 160, 192, 256};
-    static_assert(sizeof(kCandidates) / sizeof(kCandidates[0]) <= kMaxTune, "report arrays");
+    constexpr int kNC = (int)(sizeof(kCandidates) / sizeof(kCandidates[0]));
+    static_assert(kNC <= kMaxTune, "report arrays");
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CK(cudaEventCreate(&e0), "event");
     CK(cudaEventCreate(&e1), "event");
     const int saved_graph = s->graph_steps, saved_seg = s->seg;
     s->graph_steps = 0;                      // time the launches themselves
-    constexpr int kNC = (int)(sizeof(kCandidates) / sizeof(kCandidates[0]));
-    constexpr int kRounds = 2;               // each candidate's best of two rounds
-    float cand_ms[kNC] = {};
-    int best = s->seg;
-    float best_ms = 0.f;
+    // one timing of a height (0: by the batch's size), kept if it is the height's best so far
+    const auto time_rows = [&](int rows, float& best) -> int {
+        int rc = eulbfs_set_tile(s, rows);
+        if (rc == EULBFS_OK) rc = eulbfs_step(s, 1);   // rebuild + warm the work list
+        if (rc != EULBFS_OK || s->nitems == 0) return rc;   // (no items: nothing to time)
+        cudaEventRecord(e0, s->stream);
+        rc = eulbfs_step(s, steps_per_candidate);
+        cudaEventRecord(e1, s->stream);
+        if (rc != EULBFS_OK) return rc;
+        if (cudaEventSynchronize(e1) != cudaSuccess) return cuda_fail(cudaGetLastError(), "autotune timing");
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        ms /= steps_per_candidate;
+        if (best == 0.f || ms < best) best = ms;
+        return EULBFS_OK;
+    };
+    float cand_ms[kNC] = {}, rule_ms = 0.f;
     int rc = EULBFS_OK;
-    for (int round = 0; round < kRounds && rc == EULBFS_OK; ++round) {
-        for (int k = 0; k < kNC; ++k) {
-            rc = eulbfs_set_tile(s, kCandidates[k]);
-            if (rc == EULBFS_OK) rc = eulbfs_step(s, 1);   // rebuild + warm the work list
-            if (rc != EULBFS_OK) break;
-            if (s->nitems == 0) break;                     // nothing to time
-            cudaEventRecord(e0, s->stream);
-            rc = eulbfs_step(s, steps_per_candidate);
-            cudaEventRecord(e1, s->stream);
-            if (rc != EULBFS_OK) break;
-            if (cudaEventSynchronize(e1) != cudaSuccess) { rc = cuda_fail(cudaGetLastError(), "autotune timing"); break; }
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            ms /= steps_per_candidate;
-            if (cand_ms[k] == 0.f || ms < cand_ms[k]) cand_ms[k] = ms;
-        }
+    for (int k = 0; k < kNC && rc == EULBFS_OK; ++k) rc = time_rows(kCandidates[k], cand_ms[k]);
+    // second round: the two slowest of the first give their steps to the rule
+    int slow[2] = {0, 1};
+    if (cand_ms[1] > cand_ms[0]) std::swap(slow[0], slow[1]);
+    for (int k = 2; k < kNC; ++k) {
+        if (cand_ms[k] > cand_ms[slow[0]]) { slow[1] = slow[0]; slow[0] = k; }
+        else if (cand_ms[k] > cand_ms[slow[1]]) slow[1] = k;
     }
+    for (int k = 0; k < kNC && rc == EULBFS_OK; ++k) {
+        if (k == slow[0] || k == slow[1]) rc = time_rows(0, rule_ms);
+        else rc = time_rows(kCandidates[k], cand_ms[k]);
+    }
+    int best = saved_seg ? saved_seg : kDefaultRows;
+    float best_ms = 0.f;
     s->tune_n = 0;
     for (int k = 0; k < kNC; ++k) {
         if (cand_ms[k] > 0.f && (best_ms == 0.f || cand_ms[k] < best_ms)) { best_ms = cand_ms[k]; best = kCandidates[k]; }
@@ -937,7 +964,7 @@ int eulbfs_autotune(eulbfs_solver* s, int steps_per_candidate, int* best_rows, f
         eulbfs_set_tile(s, saved_seg);
         return fail(rc, msg.c_str());
     }
-    eulbfs_set_tile(s, best);
+    eulbfs_set_tile(s, best_ms == 0.f ? saved_seg : rule_ms > 0.f && rule_ms <= best_ms ? 0 : best);
     if (best_rows) *best_rows = best;
     if (best_ms_per_step) *best_ms_per_step = best_ms;
     return EULBFS_OK;

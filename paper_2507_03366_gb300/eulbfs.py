@@ -113,6 +113,7 @@ SIGNATURES = [
     ("eulbfs_use_graphs", ct.c_int, [ct.c_void_p, ct.c_int]),
     ("eulbfs_autotune", ct.c_int, [ct.c_void_p, ct.c_int, ct.POINTER(ct.c_int), ct.POINTER(ct.c_float)]),
     ("eulbfs_set_tile", ct.c_int, [ct.c_void_p, ct.c_int]),
+    ("eulbfs_work_list", ct.c_int, [ct.c_void_p] + [ct.POINTER(ct.c_int)] * 4),
     ("eulbfs_set_tile_wait_probe", ct.c_int, [ct.c_void_p, ct.c_int]),
     ("eulbfs_autotune_report", ct.c_int, [ct.c_void_p, ct.POINTER(ct.c_int), ct.POINTER(ct.c_float), ct.c_int,
                                           ct.POINTER(ct.c_int)]),
@@ -293,8 +294,15 @@ class Solver:
     def set_tile(self, tile_y: int):
         _check(lib().eulbfs_set_tile(self._h, tile_y))
 
+    def work_list(self) -> dict:
+        """What the next step runs: the kernel, the target height, and how many work items."""
+        v = [ct.c_int() for _ in range(4)]
+        _check(lib().eulbfs_work_list(self._h, *[ct.byref(x) for x in v]))
+        return dict(zip(("short_items", "rows", "items", "ctas_per_sm"), (x.value for x in v)))
+
     def autotune(self, steps_per_candidate: int = 10):
-        """Time the work-item heights on the live batch; returns (rows, ms per step)."""
+        """Time the work-item heights on the live batch; returns the fastest (rows, ms per step).
+        The solver takes it unless the heights by the batch's size are faster."""
         rows, ms = ct.c_int(), ct.c_float()
         _check(lib().eulbfs_autotune(self._h, steps_per_candidate, ct.byref(rows), ct.byref(ms)))
         return rows.value, ms.value
