@@ -74,10 +74,12 @@ __device__ __forceinline__ void two_sum(R a, R b, R& s, R& e) {
 // as their bits.  With the update's shorter first stage and the radii kept per
 // column, FP64 us per step, bound by that pipe: 16 domains 4913 -> 4710, 256^2
 // 290 -> 279, 512^2 917 -> 880, 256x4 47.1 -> 45.3.
-constexpr long long kBitsOne = 0x3ff0000000000000LL, kBitsInf = 0x7ff0000000000000LL;
+// (Unsigned: the difference wraps for zeros and negative numbers.)
+constexpr unsigned long long kBitsOne = 0x3ff0000000000000ULL, kBitsInf = 0x7ff0000000000000ULL;
+__device__ __forceinline__ unsigned long long bits_of(double x) { return (unsigned long long)__double_as_longlong(x); }
 __device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
 __device__ __forceinline__ bool positive(double x) {
-    return (unsigned long long)(__double_as_longlong(x) - 1) < (unsigned long long)kBitsInf;
+    return bits_of(x) - 1 < kBitsInf;
 }
 __device__ __forceinline__ bool negative(float x) { return x < 0.0f; }
 __device__ __forceinline__ bool negative(double x) { return positive(-x); }
@@ -86,7 +88,7 @@ __device__ __forceinline__ bool is_finite(double x) { return (__double2hiint(x) 
 
 __device__ __forceinline__ float clamp01(float c) { return c < 0.0f ? 0.0f : (c > 1.0f ? 1.0f : c); }
 __device__ __forceinline__ double clamp01(double c) {
-    const bool above = (unsigned long long)(__double_as_longlong(c) - kBitsOne - 1) < (unsigned long long)(kBitsInf - kBitsOne);
+    const bool above = bits_of(c) - (kBitsOne + 1) < kBitsInf - kBitsOne;
     return negative(c) ? 0.0 : (above ? 1.0 : c);
 }
 
