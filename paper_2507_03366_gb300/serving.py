@@ -10,7 +10,8 @@ so all running cases advance together in the same stage launches:
   step   -- one eulbfs_step(chunk) advances every running case (each stops
             at its own step count, its slot leaves the work list);
   retire -- finished cases have their fields copied to the host and their
-            memory released; their time to solution is completion - arrival.
+            memory released; their time to solution is completion - arrival
+            (- admission where a closed loop admits a case before it arrives).
             A case whose own state became NaN or Inf (its per-domain flag,
             read after every chunk) is retired with that error at once.
 
@@ -41,9 +42,18 @@ class Outcome:
     error: Optional[str] = None
 
     @property
+    def start_s(self) -> float:
+        """What its times count from: its arrival, or its admission where a
+        closed loop (realtime=False) admits it before that."""
+        return min(self.arrival_s, self.admitted_s)
+
+    @property
+    def queue_s(self) -> float:
+        return self.admitted_s - self.start_s
+
+    @property
     def latency_s(self) -> float:
-        # a closed loop (realtime=False) may admit a case before its nominal arrival
-        return self.finished_s - min(self.arrival_s, self.admitted_s)
+        return self.finished_s - self.start_s
 
 
 @dataclass
@@ -69,7 +79,7 @@ class ServeReport:
                "admissions_deferred": self.rejected_busy}
         out.update(self.latency_percentiles())
         if done:
-            out["mean_queue_s"] = float(np.mean([o.admitted_s - o.arrival_s for o in done]))
+            out["mean_queue_s"] = float(np.mean([o.queue_s for o in done]))
         out.update(self.extra)
         return out
 
