@@ -365,16 +365,20 @@ struct ItemPlan {
 // sweep, so a batch that does not fill the chip is cut finer, unless
 // eulbfs_set_tile names a height (s->seg).  us per step on one GB300, FP32C unless marked; 64: the height
 // that every batch once had:
-//   - the short-item kernel, up to 4.1 items of kShortRows rows per SM: 128^2
+//   - the short-item kernel, up to 4.3 items of kShortRows rows per SM: 128^2
 //     121 (64) -> 13.9, 400x200 193 -> 21.6, 333x251 131 -> 21.6, 1024x4 27 -> 12.3;
 //     FP64 256x4 135 -> 44.7, 128^2 1281 -> 108, 256^2 1326 -> 277 (the tiled
-//     kernel in 8-row items: 31, 37, 34, 26; FP64 135, 192, 340).  At the limit
-//     the two meet: 384^2 39 (tiled 43), 448^2 53 (50); FP64 384^2 590 (611);
+//     kernel in 8-row items: 31, 37, 34, 26; FP64 135, 192, 340).  Around the
+//     limit, short and (tiled): 384^2 35.5 (36.8), 400^2 (4.28 items per SM) 37.0
+//     (37.8), 416^2 (4.79) 41.2 (39.7); (r, z) 36.3 (38.3), 37.9 (39.4), 42.2 (41.6);
+//     2540x62 (4.18) 37.0 (36.7), six domains of 128x168 (4.15) 38.6 (41.2); FP64 384^2
+//     526 (545), 400^2 548 (564), 416^2 612 (627), 448^2 704 (700).  A launch per
+//     stage: 400^2 49.7 (59.5), in two slabs 57.0 (68.7), FP64 621 (728);
 //   - else the tiled kernel with the tallest items that still make 2.6 waves of
 //     its resident CTAs, up to kDefaultRows: 512^2 54 (8 rows; 16: 58, 64: 126),
 //     640^2 70 (16; 8: 79, 64: 147), 1024^2 155 (24; 16: 164, 32: 151, 64: 208),
-//     16 droplet domains 214 (32; 24: 225, 40: 219, 64: 227), 64 domains 914 (128;
-//     160: 927, 64: 941).
+//     16 droplet domains 214 (32; 24: 225, 40: 219, 64: 227), the benchmark's 64
+//     (r, z) domains of 6.80 M cells 939 (128; 96: 944, 64: 956).
 // The height of short items: the one with the least work for the busiest SM.  An
 // item of h rows costs as b + h (a stage of one FP64 item keeps its SM's pipe
 // busy for about 8 + 9 h thousand clocks, whoever shares the SM; fitted for
@@ -419,11 +423,10 @@ bool launch_per_stage(const eulbfs_solver* s) {
 // A launch per stage ends with its last item, so where items of up to this many
 // rows make one wave of the tiled kernel's resident CTAs, the shortest such are
 // taken.  us per step of droplets in slabs, with the rule for whole-step launches and
-// in one wave: 400^2 in two 71.6 (8 rows) -> 69.4 (16), 512^2 in two 80.5 (8) -> 72.8
-// (16), 600^2 in two 99.9 (8) -> 96.9 (24), 640^2 in four 126.7 (16) -> 99.7 (24),
-// 768^2 in four 131.0 (16) -> 127.3 (32); FP64 512^2 1125 (16) -> 1087 (32).  Beyond,
-// several waves are better: 900^2 in four 176.6 (24; one wave of 48: 180.3),
-// 1024^2 in three 217 (24; 64: 241).
+// in one wave: 512^2 in two 80.5 (8 rows) -> 72.8 (16), 600^2 in two 99.9 (8) -> 96.9
+// (24), 640^2 in four 126.7 (16) -> 99.7 (24), 768^2 in four 131.0 (16) -> 127.3 (32);
+// FP64 512^2 1125 (16) -> 1087 (32).  Beyond, several waves are better: 900^2 in four
+// 176.6 (24; one wave of 48: 180.3), 1024^2 in three 217 (24; 64: 241).
 constexpr int kOneWaveRows = 32;
 
 ItemPlan plan_items(const eulbfs_solver* s) {
@@ -433,7 +436,7 @@ ItemPlan plan_items(const eulbfs_solver* s) {
     for (const Dom& d : s->doms)
         if (d.active()) strip_rows += (long long)((d.grid.nx + kStripX - 1) / kStripX) * d.grid.ny;
     // input tiles, and so the probe of their waits, are the tiled kernel's
-    if (!s->tile_probe && strip_rows * 10 <= 41LL * s->sms * kShortRows) return ItemPlan{true, short_rows(s, fp64)};
+    if (!s->tile_probe && strip_rows * 10 <= 43LL * s->sms * kShortRows) return ItemPlan{true, short_rows(s, fp64)};
     const long long resident = (long long)stage_blocks_per_sm(s->precision) * s->sms;
     if (launch_per_stage(s))
         for (int rows = kChunk; rows <= kOneWaveRows; rows += kChunk) {

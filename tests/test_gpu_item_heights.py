@@ -1,6 +1,7 @@
 """Heights of work items: eulbfs_set_tile names one and the batch runs in items
 of that height, 0 leaves it to the batch's size, and the autotuner keeps the
 better of the two."""
+import numpy as np
 import pytest
 
 from paper_2507_03366_gb300 import eulbfs
@@ -73,3 +74,32 @@ def test_work_list_arguments():
     s = eulbfs.Solver([wl.droplet(32)], precision=eulbfs.FP32C)
     assert eulbfs.lib().eulbfs_work_list(s._h, None, None, None, None) == eulbfs.OK
     assert eulbfs.lib().eulbfs_work_list(None, None, None, None, None) == eulbfs.EINVAL
+
+
+@pytest.mark.parametrize("precision", [eulbfs.FP32C, eulbfs.FP64])
+@pytest.mark.parametrize("n,short", [(384, 1), (400, 1), (416, 0)])
+def test_the_short_kernel_ends_where_the_tiled_one_is_faster(n, short, precision):
+    """4.1, 4.3 and 4.8 items of eight rows per SM; the same fields by both kernels."""
+    case = wl.droplet(n, theta_deg=82.0, St=0.25, Tw=-0.6, axisymmetric=True, hysteresis=(100.0, 39.0))
+    own, tiled = (eulbfs.Solver([case], precision=precision) for _ in range(2))
+    assert own.work_list()["short_items"] == short
+    tiled.set_tile(16)
+    for s in (own, tiled):
+        s.step(18)
+    for f in ("H", "T", "Fl", "C", "p", "u", "v"):
+        assert np.array_equal(own.fields()[f], tiled.fields()[f]), f
+
+
+def test_one_wave_of_16_rows_where_a_step_is_a_launch_per_stage():
+    """448 x 448 in two slabs: 420 items of 16 rows for 608 resident CTAs, above the short kernel's limit."""
+    case = wl.droplet(448, theta_deg=82.0, St=0.25, Tw=-0.6, axisymmetric=True, hysteresis=(100.0, 39.0))
+    split, whole = (eulbfs.Solver([], precision=eulbfs.FP32C) for _ in range(2))
+    slots = split.add_split(case, 2)
+    whole.add(case)
+    w = split.work_list()
+    assert (w["short_items"], w["rows"], w["items"]) == (0, 16, 420)
+    for s in (split, whole):
+        s.step(6)
+    a, b = split.split_fields(slots), whole.fields()
+    for f in ("H", "T", "Fl", "C", "p", "u", "v"):
+        assert np.array_equal(a[f], b[f]), f
