@@ -3,11 +3,12 @@
 // A solver holds a set of domains ("slots").  Each domain owns one device
 // allocation: its descriptor, three state buffers (W^n and the two
 // intermediate Runge-Kutta stages), F_s of the previous step and the lagged
-// dF_s/dt.  The active domains form one tile work list; a time step is three
-// launches of the stage kernel over that list (Eq. 58), optionally replayed
-// from a captured CUDA graph; each stage launch and each graph replay is an
-// NVTX range for profilers.  Domains can be added and removed between steps
-// (continuous batching) under a device-memory budget.
+// dF_s/dt.  The active domains form one work list; one launch of a stage kernel
+// runs up to 16 time steps over it, or one Runge-Kutta stage (Eq. 58) where split
+// domains exchange halos in between, optionally replayed from a captured CUDA
+// graph; each launch and each graph replay is an NVTX range for profilers.
+// Domains can be added and removed between steps (continuous batching) under a
+// device-memory budget.
 #include <cuda.h>           // CUtensorMap and its enums only: the encoder is fetched through the runtime
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>   // header-only: ranges cost a pointer test unless a profiler is attached

@@ -145,7 +145,7 @@ __device__ __forceinline__ void invert_enthalpy(const Consts<R>& K, R Hh, R Hl, 
     const R dl = pair_sum(Hh - HL, Hl);
     // one division whichever branch a cell takes: a warp with cells on several
     // branches passes it once, and the code has no divergent paths.  us per step: 64
-    // domains 1021 -> 1006, 512^2 54.1 -> 53.2, 128^2 14.0 -> 13.9; FP64 16 domains
+    // domains (7.23 M cells) 1021 -> 1006, 512^2 54.1 -> 53.2, 128^2 14.0 -> 13.9; FP64 16 domains
     // 4711 -> 4702.  (Choosing num and den by selects keeps more registers live: the
     // two-per-SM short kernel spilled 28 bytes and lost 0.5 %.)
     const bool solid = negative(ds), liquid = positive(dl);

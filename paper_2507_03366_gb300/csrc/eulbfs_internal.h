@@ -177,7 +177,7 @@ constexpr int kTmapBytes = 128;   // sizeof(CUtensorMap)
 struct StageLaunch {
     const void* consts;      // Consts<R>[ndomains] in device memory
     const void* tmaps;       // CUtensorMap[ndomains][3]: one per state buffer (used where Consts::tma)
-    const int4* items;       // (domain, strip, y0, y1), tallest first
+    const int4* items;       // (domain, strip, y0, y1), tallest first; short items in row order
     int nitems;
     int stage;               // the stage of a one-stage launch: 0, 1, 2
     int stages;              // 1: stage `stage` alone; 3 k: k whole time steps (items of stage 0, 1, 2 of the first step, then of the next)

@@ -2,7 +2,7 @@
 // of the EULBFS explicit step over every domain of a batch.
 //
 // Work decomposition.  A work item is a strip segment of one domain: 31
-// interior columns wide, `seg` rows high.  A CTA of 8 warps sweeps its segment
+// interior columns wide and a run of rows high.  A CTA of 8 warps sweeps its segment
 // upwards in chunks of 8 rows, keeping the derived fields of the rows it needs
 // in a 16-row ring buffer in shared memory, so every cell of the segment is
 // loaded and derived once per stage (plus a 3-column halo on each side and a
@@ -280,9 +280,7 @@ __device__ __forceinline__ bool load_barrier_failed(Smem<R>& S, bool ok) {
         return false;
     }
 }
-// A tile wait gave up: report it, wait (with the same bound) for the copy
-// still in flight so that it cannot land in shared memory after the CTA has
-// left, and stop.
+
 // A wait for the items an item reads gave up (whole-step launches): report
 // it as a bounded wait that gave up, wait for a prologue tile that may be in
 // flight, and stop.
@@ -293,6 +291,9 @@ __device__ __noinline__ void dep_abort(Smem<R>& S, TileIO io, int* flag) {
         if (S.pre) tile_wait(S, io);
 }
 
+// A tile wait gave up: report it, wait (with the same bound) for the copy
+// still in flight so that it cannot land in shared memory after the CTA has
+// left, and stop.
 template <class R>
 __device__ __noinline__ bool tile_abort(Smem<R>& S, TileIO io, int* flag) {
     if (threadIdx.x == 0) atomicOr(flag, 2);
@@ -444,7 +445,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 4 : 2) stage_kernel(Stage
     // start the look-up is an atomic and four dependent loads, with three more
     // barriers).  us per step, before and after: 512^2 58.9 -> 54.1, 640^2 74.9 -> 70.0,
     // 1024^2 164.3 -> 154.7, 16 domains 222 -> 214 (planar, streaming 244 -> 237),
-    // 64 domains 1041 -> 1022; FP64 unchanged (919 -> 917 at 512^2).
+    // 64 domains (7.23 M cells) 1041 -> 1022; FP64 unchanged (919 -> 917 at 512^2).
     // In a whole-step launch the items of stage 1 follow all of stage 0 and those
     // of stage 2 all of stage 1 (then stage 0 of the next step, when the
     // launch runs several), and an item waits for the items of the previous

@@ -280,9 +280,11 @@ __device__ __forceinline__ void face_value8_2(const P2<R>* f, const FaceIdx& x, 
 // Folding the weights into V and so into X, G and H takes a face from about 237
 // to 191 FP operations besides its division (against the t-points one by one and
 // each moment from its own sums).  us per step: FP64, bound by its pipe, 16
-// domains 6460 -> 5760, 256^2 348 -> 316; FP32C, bound by issue, 64 domains 1023
-// -> 977, 16 domains 260 -> 251, 512^2 63.6 -> 60.9.  Constants like 1/6 are a
-// biased 3e-8 in FP32: none stands on an undivided advective or conductive flux.
+// domains 6460 -> 5760, 256^2 348 -> 316; FP32C, bound by issue, the benchmark's 64
+// domains (6.80 M cells) 1023 -> 977, 16 domains 260 -> 251, 512^2 63.6 -> 60.9.
+// Constants like 1/6 are a biased 3e-8 in FP32: none stands on an undivided flux
+// of mass, enthalpy or phase, or on the normal momentum flux.  The tangential
+// momentum flux carries that of its 1/24, as it would that of cs^2 = 1/3.
 template <class R>
 struct SideTerms { R X, V, hd, F, G, H; };
 
@@ -733,7 +735,7 @@ __device__ __forceinline__ void cell_update(Core<R>& S, const Cell& in, int stag
         o.Cl = R(0);
     } else {
         // Eq. 58 as W^n + increment (stage 0: dt R alone, 14 operations fewer; us per
-        // step of 64 domains 1006 -> 994, 512^2 53.2 -> 52.7); H and C kept as
+        // step of 64 domains (7.23 M cells) 1006 -> 994, 512^2 53.2 -> 52.7); H and C kept as
         // compensated pairs.  TwoSum for the sum and the renormalisation keeps
         // every pair canonical.
         R dH, dC;
